@@ -98,14 +98,16 @@ enum {
   DTB_W_INT8 = 3   /* int8, w_acc = w << (weight_shift + row_shift[source]) */
 };
 
-/* How delivered events wait out their delay (the results are the same bit for bit). */
+/* How delivered events wait out their delay (the results are the same bit for bit;
+ * DTB_DELIVER_BINS without a bin_capacity of the caller's keeps the queue layout
+ * for networks whose accumulators are at most 24 MiB: it is the faster one there). */
 enum {
   DTB_DELIVER_RING = 0,  /* dense ring acc[D][n_channels][N]: every synapse event is one int32
                             reduction into slot (t + d) mod D */
-  DTB_DELIVER_QUEUE = 1, /* delay-1 events are reduced straight into a one-slot accumulator; longer
-                            ones are appended (target|class, w_acc) to the queue of their arrival
-                            step, staged per batch of work items in shared memory, and each queue
-                            is reduced into the accumulator one step before its arrival step */
+  DTB_DELIVER_QUEUE = 1, /* delay-1 events are reduced straight into a one-slot accumulator; of the
+                            longer ones the runs of synapses (a stretch of a row with one delay)
+                            wait in the queue of their arrival step, and are reduced into the
+                            accumulator one step before it */
   DTB_DELIVER_BINS = 2   /* events wait in bins by arrival step parity and target region (4096
                             neurons): delay-1 events are written straight into the bins of step
                             t + 1 (their targets lie in the source's voxel, a few regions, so a
@@ -158,15 +160,12 @@ typedef struct dtb_network_desc {
                                  0 -> 4 * event_queue_capacity / regions, at least 4096, at most
                                  event_queue_capacity; rounded up to an odd number of 128-byte lines
                                  (32 events each, 16 with DTB_W_INT32 weights) */
-  int64_t event_queue_capacity; /* DTB_DELIVER_QUEUE and _BINS: events one arrival step's queue holds,
-                                   0 .. 2^32-64; 0 -> 2N; rounded up to an odd number of 16-event
-                                   lines.  Events beyond a queue's or a bin's capacity are added into
-                                   a dense spill ring instead (exact, slower), so no capacity changes
-                                   the results.  Limit: a queue's and a bin's event counters are
-                                   32-bit, so fewer than 2^32 events may be queued for one arrival
-                                   step (and one region); more would wrap the counter and overwrite
-                                   queued events.  Only a network of more than 2^32 long-delay
-                                   synapses whose sources fire in lockstep can reach it */
+  int64_t event_queue_capacity; /* DTB_DELIVER_QUEUE and _BINS: what one arrival step's queue holds,
+                                   runs of synapses in the queue layout and events in bins,
+                                   0 .. 2^32-64; 0 -> 2N; rounded up to an odd number of 16-entry
+                                   lines (the queue layout: in each of eight parts).  What finds a
+                                   queue or a bin full is added into a dense spill ring instead
+                                   (exact, slower), so no capacity changes the results */
   void* stream;               /* cudaStream_t all work is queued on; must not be the legacy
                                  default stream (graph capture); NULL -> a library stream */
   dtb_alloc_fn alloc;         /* device allocator, or NULL */

@@ -20,7 +20,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libdtb.so")
-SOURCES = ["step_kernels.cu", "setup_kernels.cu", "standalone.cu", "standalone_noalloc.cu", "assimilate.cu",
+SOURCES = ["step_kernels.cu", "deliver.cu", "bins.cu", "setup_kernels.cu", "standalone.cu", "standalone_noalloc.cu", "assimilate.cu",
            "mlp.cu", "dtb_api.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "--fmad=false", "-Xcompiler", "-fPIC,-ffp-contract=off,-O2",

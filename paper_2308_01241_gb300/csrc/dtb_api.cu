@@ -48,7 +48,17 @@ constexpr int kTimedKernels = 5;  // update, compaction, delivery, drain or binn
 // step beside the neuron update of the next by default: their kernels leave
 // most of the GPU idle, and the step is a chain of short launches.  Larger
 // networks' updates fill every SM, and the compaction then waits its turn.
-constexpr int32_t kBesideMaxBlocks = 4096;
+// Measured at 5M neurons (bins): 67.1 -> 61.2 us a step at 7 Hz, 106.2 -> 104.5
+// at 30 Hz; at 20M it was 4 % slower.
+constexpr int32_t kBesideMaxBlocks = 6144;
+// Networks whose accumulator (4 bytes per neuron and channel) is at most this
+// large use the queue layout where bins are asked for (without a bin capacity
+// of the caller's): it stays in the L2 cache beside the neuron state, and one
+// reduction there per event is less work than sorting the events into bins.
+// Step, bins -> queue: 33.1 -> 20.1 us (1M neurons, 15 Hz), 36.4 -> 31.6 (2M);
+// at 5M and 7 Hz the bins are ahead (61.2 against 65.7 us), their accumulator
+// no longer fits.
+constexpr int64_t kQueueMaxBytes = 24 << 20;
 constexpr int kBoldLogCap = 1024;
 
 }  // namespace
@@ -60,7 +70,7 @@ struct dtb_net {
   // side branches of the step sequence: delivery, queue drain and BOLD step
   // (fork and join by events)
   cudaStream_t side[3] = {nullptr, nullptr, nullptr};
-  cudaEvent_t ev[8] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+  cudaEvent_t ev[10] = {};
   dtb_alloc_fn alloc = nullptr;
   dtb_free_fn free_fn = nullptr;
   void* alloc_ctx = nullptr;
@@ -81,6 +91,7 @@ struct dtb_net {
   int sms = 1;
   cudaGraphExec_t graph[33] = {};  // graph[k]: a chunk of k body steps (k <= kGraphSteps), built on first use
   int64_t t = 0;           // steps run (mirror of *t_base)
+  int log_par = 0;         // the copy of the log's position that the last call left
   int64_t call_t0 = 0;     // t at the start of the last dtb_step
   int64_t call_steps = 0;  // steps of the last dtb_step
   int64_t step_off_cap = 0;
@@ -231,11 +242,11 @@ dtb_status init_state(dtb_net* net) {
   if (g.mode == dtb::kModeBins)
     DTB_CUDA(cudaMemsetAsync(g.bcnt, 0, 8 * dtb::kBcntStride * 2 * (size_t)g.n_reg, st));
   if (g.mode) {
-    DTB_CUDA(cudaMemsetAsync(g.qcnt, 0, 8 * dtb::kQcntStride * (size_t)g.D, st));
-    DTB_CUDA(cudaMemsetAsync(g.drain_done, 0, 16, st));
+    DTB_CUDA(cudaMemsetAsync(g.qcnt, 0, 8 * dtb::kQcntStride * (size_t)g.D * g.n_sub, st));
     DTB_CUDA(cudaMemsetAsync(g.spill, 0, sizeof(int32_t) * (size_t)g.D * g.nch * g.npad, st));
     DTB_CUDA(cudaMemsetAsync(g.spill_dirty, 0, sizeof(int32_t) * (size_t)g.D, st));
   }
+  if (g.chunk_cnt) DTB_CUDA(cudaMemsetAsync(g.chunk_cnt, 0, 16, st));
   DTB_CUDA(cudaMemsetAsync(g.t_base, 0, sizeof(int64_t), st));
   DTB_CUDA(cudaMemsetAsync(g.events, 0, sizeof(unsigned long long), st));
   DTB_CUDA(cudaMemsetAsync(g.spikes, 0, sizeof(unsigned long long), st));
@@ -280,7 +291,7 @@ dtb_status ensure_step_off(dtb_net* net, int64_t n_steps) {
 // delivery of step t-1's spikes runs beside the neuron update of step t,
 // which does not read its arrivals (they are due at step t + 1 or later).
 // Per step, on four streams:
-//   s0: update(t) -> compact(t)                      [compact waits deliver(t-1), bold(t-1)]
+//   s0: update(t) -> compact(t)                      [compact waits deliver(t-1), bold(t-2)]
 //   s1: compact(t) -> deliver(t)
 //   s2: update(t), deliver(t-1) -> drain of the arrivals at t+1   [queue mode]
 //       update(t-1), deliver(t-2) -> binning of the arrivals at t [bins mode]
@@ -290,12 +301,16 @@ dtb_status ensure_step_off(dtb_net* net, int64_t n_steps) {
 // delay-1 events go straight into the bins, so the queue of the arrivals at t
 // is complete after deliver(t-2); update(t-1) has emptied the bins of that
 // parity.  The binning of step t thus runs beside deliver(t-1) and update(t).
-// With net->beside (small networks) the compaction moves to s1 as well:
-//   s0: update(t)                       [waits deliver(t-2) and the binning or drain above]
-//   s1: update(t), bold(t-1) -> compact(t) -> deliver(t)
+// With net->beside the compaction moves off s0:
+//   s0: update(t)                       [waits deliver(t-2), compact(t-2) and the binning or drain above]
+//   s1: update(t), bold(t-2) -> compact(t) -> deliver(t)
 // so compact(t) runs beside update(t + 1).  The two write different copies of
 // the spike bits and block counts (the step's index parity); update(t + 2)
-// reuses compact(t)'s copy only after deliver(t), which follows compact(t).
+// reuses compact(t)'s copy only after it.  In the queue mode the update lists the
+// delivery's work itself and nothing waits for the compaction (which then only
+// feeds the spike log and the BOLD step):
+//   s1: update(t) -> deliver(t)
+//   s3: update(t) -> compact(t) -> bold(t)   [with net->beside; else compact(t) on s0]
 // update(t) still consumes the arrivals at t - 1 after every delivery that
 // adds to them: deliver(t-2) for delay 1, the binning or drain for the rest.
 // Events are those of this sequence only; work before it is complete.
@@ -319,7 +334,9 @@ dtb::DevNet step_view(const dtb_net* net, int32_t t_rel) {
 
 dtb_status enqueue_range(dtb_net* net, int32_t k, bool head, cudaEvent_t* tev = nullptr, bool* ran = nullptr) {
   cudaStream_t s0 = net->stream, s1 = net->side[0], s2 = net->side[1], s3 = net->side[2];
-  cudaEvent_t evF = net->ev[0], evC = net->ev[1], evB = net->ev[2], evS = net->ev[7];
+  cudaEvent_t evF = net->ev[0], evS = net->ev[7];
+  cudaEvent_t evB[2] = {net->ev[2], net->ev[9]};  // bold(s), by parity of s
+  cudaEvent_t evC[2] = {net->ev[1], net->ev[8]};  // compact(s), by parity of s
   cudaEvent_t* evD = net->ev + 3;  // deliver(s), by parity of s
   cudaEvent_t* evR = net->ev + 5;  // drain or binning issued at step s, by parity of s
   const bool q = net->g.mode == dtb::kModeQueue, bins = net->g.mode == dtb::kModeBins;
@@ -337,7 +354,8 @@ dtb_status enqueue_range(dtb_net* net, int32_t k, bool head, cudaEvent_t* tev = 
     const bool first = head && s == 0;
     if (q && s >= 2) DTB_CUDA(cudaStreamWaitEvent(s0, evR[(s - 2) & 1], 0));
     if (bins && s >= 1) DTB_CUDA(cudaStreamWaitEvent(s0, evR[(s - 1) & 1], 0));
-    if (beside && s >= 2) DTB_CUDA(cudaStreamWaitEvent(s0, evD[(s - 2) & 1], 0));  // deliver(s-2)
+    if (s >= 2 && (beside || q)) DTB_CUDA(cudaStreamWaitEvent(s0, evD[(s - 2) & 1], 0));  // deliver(s-2)
+    if (s >= 2 && beside) DTB_CUDA(cudaStreamWaitEvent(s0, evC[(s - 2) & 1], 0));         // compact(s-2)
     if (bins) {
       if (s >= 1) DTB_CUDA(cudaStreamWaitEvent(s2, evF, 0));               // update(s-1)
       if (s >= 2) DTB_CUDA(cudaStreamWaitEvent(s2, evD[(s - 2) & 1], 0));  // deliver(s-2)
@@ -352,20 +370,19 @@ dtb_status enqueue_range(dtb_net* net, int32_t k, bool head, cudaEvent_t* tev = 
     DTB_CUDA(mark(s, 0, 1, s0));
     DTB_CUDA(cudaEventRecord(evF, s0));
     // the compaction: after the update on s0, or beside the next update on s1
-    // (there deliver(s-1) precedes it on its own stream)
-    cudaStream_t sc = beside ? s1 : s0;
-    if (beside) DTB_CUDA(cudaStreamWaitEvent(s1, evF, 0));
-    if (s >= 1) {
-      if (!beside) DTB_CUDA(cudaStreamWaitEvent(s0, evD[(s - 1) & 1], 0));
-      DTB_CUDA(cudaStreamWaitEvent(sc, evB, 0));
-    }
+    // (there deliver(s-1) precedes it on its own stream) or, in the queue mode, s3
+    cudaStream_t sc = !beside ? s0 : q ? s3 : s1;
+    if (beside) DTB_CUDA(cudaStreamWaitEvent(sc, evF, 0));
+    if (s >= 1 && !beside && !q) DTB_CUDA(cudaStreamWaitEvent(s0, evD[(s - 1) & 1], 0));
+    if (s >= 2) DTB_CUDA(cudaStreamWaitEvent(sc, evB[(s - 2) & 1], 0));
     DTB_CUDA(mark(s, 1, 0, sc));
-    DTB_CUDA(dtb::launch_spike_compact(step_view(net, s), s, sc, first ? 1 : -1));
+    DTB_CUDA(dtb::launch_spike_compact(step_view(net, s), s, sc));
     DTB_CUDA(mark(s, 1, 1, sc));
-    DTB_CUDA(cudaEventRecord(evC, sc));
-    if (!beside) DTB_CUDA(cudaStreamWaitEvent(s1, evC, 0));
+    DTB_CUDA(cudaEventRecord(evC[s & 1], sc));
+    if (q) DTB_CUDA(cudaStreamWaitEvent(s1, evF, 0));
+    else if (!beside) DTB_CUDA(cudaStreamWaitEvent(s1, evC[s & 1], 0));
     DTB_CUDA(mark(s, 2, 0, s1));
-    DTB_CUDA(dtb::launch_spike_deliver(net->g, s, net->deliver_blocks, s1));
+    DTB_CUDA(dtb::launch_spike_deliver(step_view(net, s), s, net->deliver_blocks, s1));
     DTB_CUDA(mark(s, 2, 1, s1));
     DTB_CUDA(cudaEventRecord(evD[s & 1], s1));
     if (q) {
@@ -376,16 +393,16 @@ dtb_status enqueue_range(dtb_net* net, int32_t k, bool head, cudaEvent_t* tev = 
       DTB_CUDA(mark(s, 3, 1, s2));
       DTB_CUDA(cudaEventRecord(evR[s & 1], s2));
     }
-    DTB_CUDA(cudaStreamWaitEvent(s3, evC, 0));
+    DTB_CUDA(cudaStreamWaitEvent(s3, evC[s & 1], 0));
     DTB_CUDA(mark(s, 4, 0, s3));
     DTB_CUDA(dtb::launch_bold_step(net->g, s, s3));
     DTB_CUDA(mark(s, 4, 1, s3));
-    DTB_CUDA(cudaEventRecord(evB, s3));
+    DTB_CUDA(cudaEventRecord(evB[s & 1], s3));
   }
   // join every branch into s0
   if (k >= 1) {
     DTB_CUDA(cudaStreamWaitEvent(s0, evD[(k - 1) & 1], 0));
-    DTB_CUDA(cudaStreamWaitEvent(s0, evB, 0));
+    DTB_CUDA(cudaStreamWaitEvent(s0, evB[(k - 1) & 1], 0));
     if (q) {
       DTB_CUDA(cudaStreamWaitEvent(s0, evR[(k - 1) & 1], 0));
       if (k >= 2) DTB_CUDA(cudaStreamWaitEvent(s0, evR[(k - 2) & 1], 0));
@@ -649,6 +666,9 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
   g.bold_cap = kBoldLogCap;
   g.log_cap = d->spike_log_capacity > 0 ? d->spike_log_capacity : ((int64_t)1 << 25);
   g.mode = d->delivery_mode;
+  if (g.mode == dtb::kModeBins && n <= (int64_t)dtb::kMaxRegions * dtb::kRegionNeurons && d->bin_capacity == 0 &&
+      4 * npad * g.nch <= kQueueMaxBytes)
+    g.mode = dtb::kModeQueue;
   g.ou = d->ou_enable ? 1 : 0;
   net->ou_mu = d->ou_mu;
   if (g.ou) {
@@ -660,9 +680,11 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
   if (g.mode) {
     int64_t cap = d->event_queue_capacity > 0 ? d->event_queue_capacity : 2 * n;
     cap = std::max<int64_t>(cap, 1024);
-    // a multiple of 16 events (the drain reads two events per 16 bytes) and an
-    // odd number of 128-byte lines, so that the queues' tails do not all map to
-    // the same L2 sets (a power-of-two stride between queues did)
+    g.n_sub = g.mode == dtb::kModeQueue ? dtb::kSubQueues : 1;
+    cap = (cap + g.n_sub - 1) / g.n_sub;
+    // an odd number of 128-byte lines of 16 run records, so that the queues'
+    // tails do not all map to the same L2 sets (a power-of-two stride between
+    // queues did)
     int64_t qc = (cap + 15) & ~(int64_t)15;
     if (((qc / 16) & 1) == 0) qc += 16;
     g.qcap = qc;
@@ -704,9 +726,8 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
     g.bcnt = (unsigned long long*)A((size_t)8 * dtb::kBcntStride * 2 * g.n_reg);
   }
   if (g.mode) {
-    g.q = (uint2*)A((size_t)8 * g.D * g.qcap);
-    g.qcnt = (unsigned long long*)A((size_t)8 * dtb::kQcntStride * g.D);
-    g.drain_done = (uint32_t*)A(16);
+    g.q = (unsigned long long*)A((size_t)8 * g.D * g.n_sub * g.qcap);
+    g.qcnt = (unsigned long long*)A((size_t)8 * dtb::kQcntStride * g.D * g.n_sub);
     g.spill = (int32_t*)A((size_t)4 * g.D * g.nch * npad);
     g.spill_dirty = (int32_t*)A((size_t)4 * g.D);
   }
@@ -725,7 +746,8 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
   g.blk_cnt = (int32_t*)A(8 * (size_t)net->cnt_par);
   g.blk_items = (int32_t*)A(8 * (size_t)net->cnt_par);
   g.n_items = (int32_t*)A(16);
-  g.spk = (int32_t*)A(4 * npad);
+  g.spk = (int32_t*)A(8 * npad);  // two copies, as the counts and the log's position
+  g.spk_par = npad;
   g.n_spk = (int32_t*)A(16);
   g.t_base = (int64_t*)A(16);
   g.log_ids = (int32_t*)A(4 * g.log_cap);
@@ -806,14 +828,21 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
   }
 
   // delivery work items: at most one per spike plus one per kItemEvents synapses
+  // (queue mode: chunks, listed by the neuron update)
   {
     const int64_t cap = n + nnz / dtb::kItemEvents + 1;
     if (cap >= ((int64_t)1 << 31)) {
       delete net;
       return fail(DTB_EINVAL, "too many delivery work items for int32 counts");
     }
-    g.items = (dtb::WorkItem*)net->dalloc(sizeof(dtb::WorkItem) * (size_t)cap);
-    if (!g.items) {
+    if (g.mode == dtb::kModeQueue) {
+      g.list_cap = (cap + 63) & ~(int64_t)63;
+      g.chunk_list = (uint32_t*)net->dalloc(4 * 2 * (size_t)g.list_cap);
+      g.chunk_cnt = (uint32_t*)net->dalloc(16);
+    } else {
+      g.items = (dtb::WorkItem*)net->dalloc(sizeof(dtb::WorkItem) * (size_t)cap);
+    }
+    if (g.mode == dtb::kModeQueue ? !g.chunk_list || !g.chunk_cnt : !g.items) {
       delete net;
       return fail(DTB_ENOMEM, "delivery work items");
     }
@@ -860,10 +889,11 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
     }
   }
 
-  // queue and bins modes with 16-bit weight codes: packed synapse records
+  // queue mode, and bins mode with 16-bit weight codes: packed synapse records
   // (8 bytes each) instead of the separate delay bytes, each chunk of a row
   // sorted by delay and target, with the chunks' run tables
-  if (g.mode != dtb::kModeRing && g.wfmt != DTB_W_INT32 && nnz > 0) {
+  g.nnz = nnz;
+  if (g.mode == dtb::kModeQueue || (g.mode == dtb::kModeBins && g.wfmt != DTB_W_INT32)) {
     // first chunk of every row, from the row pointers
     std::vector<int64_t> rp((size_t)n + 1), cb((size_t)n + 1);
     cudaError_t e2 = cudaMemcpy(rp.data(), g.row_ptr, 8 * ((size_t)n + 1), cudaMemcpyDeviceToHost);
@@ -876,17 +906,21 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
     const int64_t n_chunks = cb[n];
     rp.clear();
     rp.shrink_to_fit();
-    uint2* pk = (uint2*)net->dalloc(8 * (size_t)nnz);
+    uint2* pk = (uint2*)net->dalloc(8 * ((size_t)nnz + 1));
+    uint8_t* dl = (uint8_t*)net->dalloc((size_t)std::max<int64_t>(nnz, 1));
     int64_t* d_cb = (int64_t*)net->dalloc(8 * ((size_t)n + 1));
     int64_t* d_rp = (int64_t*)net->dalloc(8 * ((size_t)n_chunks + 1));
-    int32_t* d_cnt = (int32_t*)net->dalloc(4 * (size_t)n_chunks);
-    if (!pk || !d_cb || !d_rp || !d_cnt) {
+    int32_t* d_cnt = (int32_t*)net->dalloc(4 * (size_t)std::max<int64_t>(n_chunks, 1));
+    dtb::ChunkInfo* d_ci = nullptr;
+    if (g.mode == dtb::kModeQueue)
+      d_ci = (dtb::ChunkInfo*)net->dalloc(sizeof(dtb::ChunkInfo) * (size_t)std::max<int64_t>(n_chunks, 1));
+    if (!pk || !dl || !d_cb || !d_rp || !d_cnt || (g.mode == dtb::kModeQueue && !d_ci)) {
       delete net;
       return fail(DTB_ENOMEM, "packed synapse records and run tables");
     }
     g.chunk_base = d_cb;
     e2 = cudaMemcpyAsync(d_cb, cb.data(), 8 * ((size_t)n + 1), cudaMemcpyHostToDevice, st);
-    if (e2 == cudaSuccess) e2 = dtb::launch_pack_fill(g, pk, d_cnt, st);
+    if (e2 == cudaSuccess) e2 = dtb::launch_pack_fill(g, pk, dl, d_cnt, st);
     std::vector<int32_t> cnt((size_t)n_chunks);
     if (e2 == cudaSuccess) e2 = cudaMemcpyAsync(cnt.data(), d_cnt, 4 * (size_t)n_chunks, cudaMemcpyDeviceToHost, st);
     if (e2 == cudaSuccess) e2 = cudaStreamSynchronize(st);
@@ -906,15 +940,17 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
       return fail(DTB_ENOMEM, "run tables");
     }
     e2 = cudaMemcpyAsync(d_rp, run_ptr.data(), 8 * ((size_t)n_chunks + 1), cudaMemcpyHostToDevice, st);
-    if (e2 == cudaSuccess) e2 = dtb::launch_run_fill(g, pk, d_rp, d_runs, st);
+    if (e2 == cudaSuccess) e2 = dtb::launch_run_fill(g, pk, dl, d_rp, d_runs, d_ci, st);
     if (e2 == cudaSuccess) e2 = cudaStreamSynchronize(st);
     if (e2 != cudaSuccess) {
       delete net;
       return cuda_fail(e2, "run tables");
     }
+    net->dfree(dl);
     g.syn_pack = pk;
     g.run_ptr = d_rp;
     g.runs = d_runs;
+    g.chunks = d_ci;
   } else {  // per-synapse delays (one byte each), read by delivery next to the target word
     uint8_t* sd = (uint8_t*)net->dalloc((size_t)std::max<int64_t>(nnz, 16));
     if (!sd) {
@@ -951,6 +987,15 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
     g.nitem_ok = too_long ? 0 : 1;
   }
 
+  {
+    cudaError_t e2 = dtb::prepare_step_kernels();
+    if (e2 == cudaSuccess) e2 = dtb::prepare_deliver_kernels();
+    if (e2 == cudaSuccess) e2 = dtb::prepare_bins_kernels();
+    if (e2 != cudaSuccess) {
+      delete net;
+      return cuda_fail(e2, "kernel attributes");
+    }
+  }
   dtb_status s = upload_consts(net);
   if (s == DTB_OK) s = init_state(net);
   if (s != DTB_OK) {
@@ -992,6 +1037,7 @@ dtb_status dtb_step(dtb_net* net, int64_t n_steps) {
   net->call_t0 = net->t;
   net->call_steps = n_steps;
   net->t += n_steps;
+  net->log_par = (int)(net->t & 1);
   return check_device_error(net);
 }
 
@@ -1066,6 +1112,7 @@ dtb_status dtb_step_timed(dtb_net* net, int64_t n_steps, double* ms, int64_t* la
   net->call_t0 = net->t;
   net->call_steps = n_steps;
   net->t += n_steps;
+  net->log_par = (int)(net->t & 1);
   return check_device_error(net);
 }
 
@@ -1073,7 +1120,7 @@ dtb_status dtb_get_spikes(dtb_net* net, int64_t* step_offsets, int32_t* ids, int
   if (!net || !n_out) return fail(DTB_EINVAL, "net or n_out is NULL");
   int64_t pos = 0;
   int32_t trunc = 0;
-  DTB_CUDA(cudaMemcpyAsync(&pos, net->g.log_pos, 8, cudaMemcpyDeviceToHost, net->stream));
+  DTB_CUDA(cudaMemcpyAsync(&pos, net->g.log_pos + net->log_par, 8, cudaMemcpyDeviceToHost, net->stream));
   DTB_CUDA(cudaMemcpyAsync(&trunc, net->g.log_trunc, 4, cudaMemcpyDeviceToHost, net->stream));
   DTB_CUDA(cudaStreamSynchronize(net->stream));
   *n_out = pos;
@@ -1166,42 +1213,25 @@ dtb_status dtb_set_state(dtb_net* net, const float* V, const float* j, const uin
   if (ref) DTB_CUDA(cudaMemcpyAsync(g.ref, ref, n, cudaMemcpyHostToDevice, st));
   if (ring && !g.mode)
     DTB_CUDA(cudaMemcpy2DAsync(g.ring, 4 * np, ring, 4 * n, 4 * n, (size_t)g.D * g.nch, cudaMemcpyHostToDevice, st));
-  if (ring && g.mode == dtb::kModeBins) {
+  if (ring && g.mode) {
     // the whole ring goes into the spill ring, which the neuron update adds
-    // in slot by slot; queues and bins start empty
+    // in slot by slot; queues, and the accumulator or the bins, start empty
     const size_t bytes = 4 * (size_t)g.D * g.nch * np;
-    std::vector<int32_t> dirty((size_t)g.D, 1);
+    std::vector<int32_t> dirty((size_t)g.D);
+    for (int64_t x = t; x < t + g.D; x++) dirty[(size_t)(x % g.D)] = dtb::spill_mark(x);  // the steps to come
     cudaError_t e = cudaMemsetAsync(g.spill, 0, bytes, st);
     if (e == cudaSuccess)
       e = cudaMemcpy2DAsync(g.spill, 4 * np, ring, 4 * n, 4 * n, (size_t)g.D * g.nch, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(g.spill_dirty, dirty.data(), 4 * (size_t)g.D, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(g.qcnt, 0, 8 * (size_t)dtb::kQcntStride * g.D, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(g.bcnt, 0, 8 * (size_t)dtb::kBcntStride * 2 * g.n_reg, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(g.qcnt, 0, 8 * (size_t)dtb::kQcntStride * g.D * g.n_sub, st);
+    if (e == cudaSuccess && g.mode == dtb::kModeBins)
+      e = cudaMemsetAsync(g.bcnt, 0, 8 * (size_t)dtb::kBcntStride * 2 * g.n_reg, st);
+    if (e == cudaSuccess && g.ring) e = cudaMemsetAsync(g.ring, 0, 4 * (size_t)2 * g.nch * np, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(e, "dense ring to spill ring");
-  } else if (ring && g.mode) {
-    // slot t mod D becomes the accumulator, every nonzero entry of the other
-    // slots one queued event
-    const size_t bytes = 4 * (size_t)g.D * g.nch * np;
-    int32_t* dense = (int32_t*)net->dalloc(bytes);
-    if (!dense) return fail(DTB_ENOMEM, "dense ring staging");
-    const int32_t xa = (int32_t)(t % g.D);
-    cudaError_t e = cudaMemsetAsync(dense, 0, bytes, st);
-    if (e == cudaSuccess)
-      e = cudaMemcpy2DAsync(dense, 4 * np, ring, 4 * n, 4 * n, (size_t)g.D * g.nch, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(g.ring, 0, 4 * (size_t)2 * g.nch * np, st);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(acc_view(net, t).ring, dense + (size_t)xa * g.nch * np, 4 * (size_t)g.nch * np,
-                          cudaMemcpyDeviceToDevice, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(g.qcnt, 0, 8 * (size_t)dtb::kQcntStride * g.D, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(g.spill, 0, bytes, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(g.spill_dirty, 0, 4 * (size_t)g.D, st);
-    if (e == cudaSuccess) e = dtb::launch_dense_to_queue(g, dense, xa, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    net->dfree(dense);
-    if (e != cudaSuccess) return cuda_fail(e, "dense ring to queues");
   }
+  if (g.chunk_cnt) DTB_CUDA(cudaMemsetAsync(g.chunk_cnt, 0, 16, st));
   DTB_CUDA(cudaMemcpyAsync(g.t_base, &t, 8, cudaMemcpyHostToDevice, st));
   DTB_CUDA(cudaStreamSynchronize(st));
   net->t = t;
@@ -1264,7 +1294,7 @@ dtb_status dtb_profile_steps(dtb_net* net, int64_t n_steps, double* ms) {
     DTB_CUDA(cudaEventRecord(ev[1], st));
     DTB_CUDA(dtb::launch_neuron_update(net->g, 0, st, net->update_stages, net->update_per_sm, dtb::kUpdFull));
     DTB_CUDA(cudaEventRecord(ev[2], st));
-    DTB_CUDA(dtb::launch_spike_compact(net->g, 0, st, 0));
+    DTB_CUDA(dtb::launch_spike_compact(net->g, 0, st));
     DTB_CUDA(cudaEventRecord(ev[3], st));
     DTB_CUDA(dtb::launch_spike_deliver(net->g, 0, net->deliver_blocks, st));
     DTB_CUDA(cudaEventRecord(ev[4], st));
@@ -1287,6 +1317,7 @@ dtb_status dtb_profile_steps(dtb_net* net, int64_t n_steps, double* ms) {
   net->call_t0 = net->t;
   net->call_steps = n_steps;
   net->t += n_steps;
+  net->log_par = (int)(net->t & 1);
   return check_device_error(net);
 }
 
@@ -1391,6 +1422,7 @@ dtb_status dtb_autotune(dtb_net* net, int32_t n_steps, int32_t* chosen) {
     float ms = 0;
     DTB_CUDA(cudaEventElapsedTime(&ms, e0, e1));
     net->t += n_steps;
+  net->log_par = (int)(net->t & 1);
     if (ms < best) {
       best = ms;
       win = c;
@@ -1680,6 +1712,7 @@ dtb_status dtb_assimilate(dtb_ensemble* ens, const float* bold_obs, int32_t n_tr
   net->call_t0 = t0 + (int64_t)(n_tr - 1) * T;
   net->call_steps = T;
   net->t = t0 + (int64_t)n_tr * T;
+  net->log_par = (int)(net->t & 1);
   ens->tr_count += (uint32_t)n_tr;
   ens_mirror(ens, th.data());
   return check_device_error(net);

@@ -64,19 +64,47 @@ struct __align__(16) WorkItem {
   int32_t pad;
 };
 
-// Run tables of the packed synapse records (queue and bins modes with 16-bit
-// weight codes).  Every chunk of kItemEvents synapses of a row is sorted at
-// creation by delay, then target; a run is a maximal stretch of one chunk
-// whose events wait in one place: the queue of one arrival step (delay d > 1,
-// key d) or, for delay 1, the bin of one target region (key kRunRegion |
-// region; in the event-queue mode every delay-1 event has key kRunRegion).
-// A run record is key | start << 14 | (length - 1) << 23, and each packed
-// record carries its run's index within the chunk in bits 16-24 of its
-// second word (the weight code stays in bits 0-15).
+// Run tables of the packed synapse records (queue mode, and bins mode with
+// 16-bit weight codes).  Every chunk of kItemEvents synapses of a row is sorted
+// at creation by delay, then target; a run is a stretch of one chunk whose
+// events wait in one place: the queue of one arrival step (delay d > 1, key d)
+// or, for delay 1, the bin of one target region (key kRunRegion | region; in
+// the queue mode every delay-1 event has key kRunRegion).  A run record is
+// key | start << 14 | (length - 1) << 23.
+//   Queue mode: a packed record is (word, accumulator value), runs of longer
+//   delays are cut at kMaxRun synapses, and what waits in a queue is the place
+//   and length of a run (run_desc), not its events.
+//   Bins mode: a packed record is (word, weight code | index of its run in the
+//   chunk << 16), and queues hold events (word, weight code).
+constexpr int kMaxRun = 64;
+// Queue mode: what the delivery of a chunk starts from, one 16-byte load: its
+// first synapse, how many there are, how many have delay 1 (they come first),
+// and its run records.
+struct __align__(16) ChunkInfo {
+  unsigned long long rec;   // first packed record | synapses << 44 | delay-1 synapses << 54 (10 bits each)
+  unsigned long long runs;  // first run record | run records << 44
+};
+__host__ __device__ __forceinline__ ChunkInfo chunk_info(int64_t e0, int len, int n1, int64_t rp0, int nr) {
+  return {(unsigned long long)e0 | (unsigned long long)len << 44 | (unsigned long long)n1 << 54,
+          (unsigned long long)rp0 | (unsigned long long)nr << 44};
+}
+constexpr unsigned long long kLow44 = (1ull << 44) - 1;
+// Queue mode: a step's queue is kSubQueues queues, each with its own counter,
+// so that the deliveries' reservations do not meet on one address.
+constexpr int kSubQueues = 8;
 constexpr uint32_t kRunRegion = 1u << 13;
+constexpr uint32_t kRunNone = 0xFFFFFFFFu;  // no run: a start and length that no chunk holds
 __host__ __device__ __forceinline__ uint32_t run_key(uint32_t r) { return r & 0x3FFFu; }
 __host__ __device__ __forceinline__ int run_start(uint32_t r) { return (int)((r >> 14) & 511u); }
 __host__ __device__ __forceinline__ int run_len(uint32_t r) { return (int)(r >> 23) + 1; }
+// A queued run: index of its first packed record, and its length (1 .. 512).
+__host__ __device__ __forceinline__ unsigned long long run_desc(int64_t first, int len) {
+  return (unsigned long long)first | (unsigned long long)len << 48;
+}
+__host__ __device__ __forceinline__ int64_t desc_first(unsigned long long d) {
+  return (int64_t)(d & ((1ull << 48) - 1));
+}
+__host__ __device__ __forceinline__ int desc_len(unsigned long long d) { return (int)(d >> 48); }
 
 // Per-voxel constants of the Euler map, 80 bytes.
 struct __align__(16) VoxConst {
@@ -120,19 +148,27 @@ struct DevNet {
   const void* w;
   const uint8_t* row_shift;
   const uint8_t* syn_delay;  // [nnz] delay of each synapse, filled once from the voxel-pair table
-  // queue and bins modes with 16-bit weight codes: each synapse packed into
-  // one 8-byte record (word, weight code | run index << 16), each chunk of a
-  // row sorted by delay and target, so that delivery reads a synapse with one
-  // load; NULL otherwise (syn_delay is used then)
+  // queue mode, and bins mode with 16-bit weight codes: the packed synapse
+  // records (see kRunRegion above); queue mode: record nnz has weight 0
   const uint2* syn_pack;
+  int64_t nnz;
   const int64_t* chunk_base;  // [n+1] first chunk of each row (with syn_pack)
   const int64_t* run_ptr;     // [chunks+1] first run of each chunk
+  // queue mode: the chunks, and the list of those whose neurons fired, in no
+  // order, that the neuron update leaves for the delivery.  Steps alternate
+  // between two lists of list_cap entries; the counts are at t mod 3 (the update
+  // of step t clears the next step's, which the delivery of step t - 2 read)
+  const ChunkInfo* chunks;
+  uint32_t* chunk_list;
+  uint32_t* chunk_cnt;
+  int64_t list_cap;
   const uint32_t* runs;       // run records
   // per-step scratch
   uint32_t* flags;
   int32_t* blk_cnt;
-  int32_t* spk;
+  int32_t* spk;     // [2][spk_par] by step parity, as n_spk and log_pos
   int32_t* n_spk;
+  int64_t spk_par;
   // delivery work items of the current step, ascending by source; blk_items
   // [nblk] per-block counts, n_items their total
   int32_t* blk_items;
@@ -152,15 +188,17 @@ struct DevNet {
   // bit 1 = an event queue overflowed
   int32_t* err;
   // delivery mode: 0 = dense ring (ring is [D][nch][npad]); 1 = event queues
-  // (ring is the one-slot accumulator [nch][npad]; q [D][qcap] entries
-  // (target | class << 30, w_acc) waiting for their arrival step, qcnt [D])
+  // (ring is the two accumulators [2][nch][npad] by step parity; q
+  // [D][kSubQueues][qcap] runs of packed synapse records (run_desc) waiting for
+  // their arrival step, qcnt [D][kSubQueues] their counts; the neuron update that
+  // consumes a step's arrivals empties its queues).  Bins mode: one queue a step
   int32_t mode;
-  int64_t qcap;
-  uint2* q;
-  unsigned long long* qcnt;  // queue x's count at qcnt[x * kQcntStride]: one L2 line per counter
-  uint32_t* drain_done;  // blocks of the current drain that finished (the last one resets the queue)
-  // bins mode (mode 2): queued events carry the synapse's weight code (see
-  // weight_code), not its accumulator value.  bins [2][n_reg][bcap] events of
+  int32_t n_sub;  // queues per arrival step
+  int64_t qcap;   // entries of one
+  unsigned long long* q;
+  unsigned long long* qcnt;  // count of queue x at qcnt[x * kQcntStride]: one L2 line per counter
+  // bins mode (mode 2): q holds events (target | class << 30, weight code; see
+  // weight_code).  bins [2][n_reg][bcap] events of
   // one arrival step, by step parity and target region, 1 word each
   // (local target | class << 12 | code << 16) or, with int32 weights, 2 words
   // (local target | class << 12, code); bcnt [2][n_reg][kBcntStride] their counts
@@ -168,9 +206,12 @@ struct DevNet {
   unsigned long long* bcnt;
   int64_t bcap;
   int32_t n_reg, ev8;
-  // event-queue mode: events that find their queue full are added into this
-  // dense ring [D][nch][npad] instead (exact int32 adds), and spill_dirty[x]
-  // tells the neuron update of the step congruent to x to consume slot x too
+  // queue and bins modes: events that find their queue or bin full are added
+  // into this dense ring [D][nch][npad] instead (exact int32 adds), and
+  // spill_dirty[x] names the arrival step of slot x's spilled events (plus one,
+  // 32 bits; see spill_mark): the neuron update of that step consumes slot x
+  // too.  A mark of an earlier step matches no later one, so none is cleared
+  // while deliveries run.
   int32_t* spill;
   int32_t* spill_dirty;
   // counters
@@ -286,7 +327,7 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t phase,
   return true;
 }
 
-// Bins mode: the stored weight of a synapse as a code that a queued event
+// Bins mode: the stored weight of a synapse as a code that its packed record
 // carries, and its accumulator value.  The code is the stored bits (int16,
 // int32, bf16) or, for int8, the byte and its total shift (8 + 5 bits), so
 // decode_weight(code) equals the weight the other modes add, bit for bit.
@@ -303,6 +344,8 @@ __device__ __forceinline__ int32_t decode_weight(uint32_t code, int32_t wfmt, in
   if (wfmt == 2) return __float2int_rn(__fmul_rn(__uint_as_float(code << 16), 65536.0f));
   return (int32_t)(signed char)(code & 0xFFu) * (1 << (code >> 8));
 }
+
+__host__ __device__ __forceinline__ int32_t spill_mark(int64_t arrival) { return (int32_t)(uint32_t)(arrival + 1); }
 
 // Voxel of neuron i: coarse table entry, then a forward scan of voxel starts.
 __device__ __forceinline__ int32_t voxel_of(const DevNet& g, int32_t i) {

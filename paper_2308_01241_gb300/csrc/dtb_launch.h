@@ -13,9 +13,11 @@ namespace dtb {
 // blocks_per_sm: resident CTAs per SM of the persistent grid (0 = as many as fit).
 cudaError_t launch_neuron_update(const DevNet& g, int32_t t_rel, cudaStream_t st, int stages, int blocks_per_sm,
                                  int32_t upd);
-cudaError_t launch_spike_compact(const DevNet& g, int32_t t_rel, cudaStream_t st, int32_t spill_rel);
+cudaError_t launch_spike_compact(const DevNet& g, int32_t t_rel, cudaStream_t st);
 cudaError_t launch_spill_clear(const DevNet& g, int32_t t_rel, cudaStream_t st);
 cudaError_t launch_spike_deliver(const DevNet& g, int32_t t_rel, int blocks, cudaStream_t st);
+// Bins mode: the delivery.
+cudaError_t launch_bins_deliver(const DevNet& g, int32_t t_rel, int blocks, cudaStream_t st);
 cudaError_t launch_drain(const DevNet& g, int32_t t_rel, int blocks, cudaStream_t st);
 // Bins mode: the queue of arrival step t + t_rel sorted into region bins.
 cudaError_t launch_bin(const DevNet& g, int32_t t_rel, cudaStream_t st);
@@ -23,6 +25,10 @@ cudaError_t launch_bold_step(const DevNet& g, int32_t t_rel, cudaStream_t st);
 cudaError_t launch_advance(const DevNet& g, int32_t k, cudaStream_t st);
 cudaError_t launch_begin_call(const DevNet& g, cudaStream_t st);
 int deliver_blocks_per_sm();
+// Attributes of the step's kernels on the current device (once per network).
+cudaError_t prepare_step_kernels();
+cudaError_t prepare_deliver_kernels();
+cudaError_t prepare_bins_kernels();
 
 // setup
 cudaError_t launch_init_voltage(const DevNet& g, uint64_t init_seed, cudaStream_t st);
@@ -37,7 +43,7 @@ cudaError_t launch_ring_gather(const DevNet& g, const int64_t* idx, int64_t m, i
 size_t compact_scratch_bytes(int64_t n);
 cudaError_t compact_bits(const uint32_t* bits, int64_t n, int32_t* ids, int32_t* count, void* scratch,
                          cudaStream_t st);
-// Event-queue mode: dense ring view <-> queues (x_acc = the accumulator's slot).
+// Queue and bins modes: the queued runs in the dense ring view (x_acc = the accumulator's slot, or -1).
 cudaError_t launch_queue_to_dense(const DevNet& g, int32_t* dense, int32_t x_acc, cudaStream_t st);
 cudaError_t launch_add(int32_t* dst, const int32_t* src, int64_t n, cudaStream_t st);
 // Bins mode: adds the bins of step x (parity x mod 2, ring slot x mod D) into
@@ -45,7 +51,6 @@ cudaError_t launch_add(int32_t* dst, const int32_t* src, int64_t n, cudaStream_t
 // the neurons whose row map [n] gives (-1: not requested); NULL skips a view.
 cudaError_t launch_bins_view(const DevNet& g, int64_t x, int32_t* dense, unsigned long long* sums,
                              const int32_t* map, int32_t* out, cudaStream_t st);
-cudaError_t launch_dense_to_queue(const DevNet& g, const int32_t* dense, int32_t x_acc, cudaStream_t st);
 // Test hook: unused queue and bin entries filled with weight-0 placeholders, counts set to value.
 cudaError_t launch_preset_counters(const DevNet& g, unsigned long long value, cudaStream_t st);
 cudaError_t launch_queue_sums(const DevNet& g, unsigned long long* sums, int32_t x_acc, cudaStream_t st);
@@ -55,13 +60,16 @@ cudaError_t launch_queue_gather(const DevNet& g, const int64_t* idx, int64_t m, 
 int32_t set_last_error(int32_t code, const std::string& msg);
 // Fills the per-synapse delay bytes out [nnz] (after the synapse check).
 cudaError_t launch_delay_fill(const DevNet& g, uint8_t* out, cudaStream_t st);
-// Fills the packed synapse records out [nnz] (queue and bins modes, weight formats
-// with 16-bit codes), after the synapse check, each chunk of a row sorted by
-// delay and target; counts [chunks] receives each chunk's number of runs
-// (g.chunk_base set).
-cudaError_t launch_pack_fill(const DevNet& g, uint2* out, int32_t* counts, cudaStream_t st);
-// The chunks' run records from the run pointers, and each record's run index.
-cudaError_t launch_run_fill(const DevNet& g, uint2* pack, const int64_t* run_ptr, uint32_t* runs, cudaStream_t st);
+// Fills the packed synapse records out [nnz + 1] (queue mode, and bins mode
+// with 16-bit weight codes), after
+// the synapse check, each chunk of a row sorted by delay and target; delays
+// [nnz] receives the records' delays, counts [chunks] each chunk's number of
+// runs (g.chunk_base set).
+cudaError_t launch_pack_fill(const DevNet& g, uint2* out, uint8_t* delays, int32_t* counts, cudaStream_t st);
+// The chunks' run records from the run pointers (and, in bins mode, each
+// packed record's run index; info, when given: the chunks' info).
+cudaError_t launch_run_fill(const DevNet& g, uint2* pack, const uint8_t* delays, const int64_t* run_ptr,
+                            uint32_t* runs, ChunkInfo* info, cudaStream_t st);
 cudaError_t launch_bounded_wait(long long max_cycles, int32_t arrive, int32_t* status, cudaStream_t st);
 cudaError_t launch_item_count(const DevNet& g, uint8_t* out, int32_t* too_long, cudaStream_t st);
 cudaError_t launch_philox(const uint32_t* ctr, const uint32_t* key, uint32_t* out, int64_t n, cudaStream_t st);

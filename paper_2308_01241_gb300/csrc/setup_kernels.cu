@@ -105,18 +105,6 @@ __global__ void delay_fill_kernel(DevNet g, uint8_t* out) {
   }
 }
 
-// Sort key of a packed record (word = target | class << 30, y = weight code |
-// delay << 16): delay, then target, then class and code.  It is a lossless
-// repacking, so the record is recovered from the key.
-__device__ __forceinline__ unsigned long long record_key(uint32_t wd, uint32_t y) {
-  return ((unsigned long long)(y >> 16) << 48) | ((unsigned long long)(wd & 0x3FFFFFFFu) << 18) |
-         ((unsigned long long)(wd >> 30) << 16) | (unsigned long long)(y & 0xFFFFu);
-}
-__device__ __forceinline__ uint2 key_record(unsigned long long k) {
-  return make_uint2((uint32_t)((k >> 18) & 0x3FFFFFFFu) | ((uint32_t)((k >> 16) & 3u) << 30),
-                    (uint32_t)(k & 0xFFFFu) | ((uint32_t)(k >> 48) << 16));
-}
-
 // Bitonic sort of 32 * R keys held by one warp, element i = r * 32 + lane in
 // register r of lane `lane`: distances below 32 exchange across lanes,
 // larger ones inside a lane.  Ascending.
@@ -152,28 +140,49 @@ __device__ __forceinline__ void warp_bitonic_sort(unsigned long long (&v)[R], in
   }
 }
 
-// Run key of a packed record (word, code | delay << 16): the arrival step's
-// queue for delay d > 1, the target region's bin for delay 1 in bins mode
-// (every delay-1 event shares one key in the event-queue mode).
-__device__ __forceinline__ uint32_t record_run_key(uint2 rec, bool bins) {
-  const uint32_t d = (rec.y >> 16) & 0xFFu;
+// Run key of a synapse: the arrival step's queue for delay d > 1, the target
+// region's bin for delay 1 in bins mode (every delay-1 event shares one key in
+// the event-queue mode).
+__device__ __forceinline__ uint32_t synapse_run_key(uint32_t word, uint32_t d, bool bins) {
   if (d > 1) return d;
-  return bins ? (kRunRegion | ((rec.x & 0x3FFFFFFFu) >> kRegionShift)) : kRunRegion;
+  return bins ? (kRunRegion | ((word & 0x3FFFFFFFu) >> kRegionShift)) : kRunRegion;
 }
 
-// Warp per row: the packed record of every synapse, (word, weight code |
-// delay << 16), the delay from the voxel-pair table.  Each chunk of
-// kItemEvents synapses (one delivery work item) is then sorted by delay and
-// target, so that its events wait in few places (runs), and the chunk's run
-// count goes to counts[chunk_base[row] + k].  The order of a row's synapses
-// changes no result: the sums are exact integers.
+// Heads of a chunk's runs, one 32-element round of a warp after the other: an
+// element starts a run when its key differs from its left neighbour's, or in
+// the queue mode when the run of a longer delay reaches kMaxRun elements.
+struct RunHeads {
+  uint32_t last = 0xFFFFFFFFu;  // key of the element before this round
+  int start = 0;                // where the run that reaches into this round began
+  __device__ __forceinline__ unsigned round(uint32_t k, bool valid, int pos, int lane, bool split) {
+    uint32_t left = __shfl_up_sync(0xFFFFFFFFu, k, 1);
+    if (lane == 0) left = last;
+    const unsigned diff = __ballot_sync(0xFFFFFFFFu, valid && k != left);
+    const unsigned mine = diff & (0xFFFFFFFFu >> (31 - lane));
+    const int from = mine ? pos - lane + 31 - __clz(mine) : start;  // first element of my stretch of one key
+    const bool cut = split && valid && !(k & kRunRegion) && (pos - from) % kMaxRun == 0;
+    const unsigned heads = diff | __ballot_sync(0xFFFFFFFFu, cut);
+    last = __shfl_sync(0xFFFFFFFFu, k, 31);
+    start = __shfl_sync(0xFFFFFFFFu, from, 31);
+    return heads;
+  }
+};
+
+// Warp per row: every synapse as a packed record, each chunk of kItemEvents
+// synapses (one delivery work item) sorted by delay (from the voxel-pair
+// table) and target, so that its events wait in few places (runs).  delays
+// receives the sorted records' delays and counts[chunk_base[row] + k] the
+// chunk's runs.  A sort key is delay | target | class | weight code, or for
+// 32-bit weights the place in the chunk, from which the weight is read again.
+// The order of a row's synapses changes no result: the sums are exact integers.
 template <int WFMT>
-__global__ void __launch_bounds__(256) pack_fill_kernel(DevNet g, uint2* out, int32_t* counts) {
+__global__ void __launch_bounds__(256) pack_fill_kernel(DevNet g, uint2* out, uint8_t* delays, int32_t* counts) {
   constexpr int R = kItemEvents / 32;
   const int lane = threadIdx.x & 31;
   const bool bins = g.mode == kModeBins;
   const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  if (gw == 0 && lane == 0) out[g.nnz] = make_uint2(0u, 0u);
   for (int64_t s = gw; s < g.n; s += nw) {
     const uint8_t* drow = g.delay + (int64_t)voxel_of(g, (int32_t)s) * g.nv;
     const int shift = WFMT == 3 ? g.wshift + (g.row_shift ? g.row_shift[s] : 0) : g.wshift;
@@ -188,23 +197,28 @@ __global__ void __launch_bounds__(256) pack_fill_kernel(DevNet g, uint2* out, in
         if (e < r1) {
           const uint32_t wd = g.word[e];
           const uint32_t d = drow[voxel_of(g, (int32_t)(wd & 0x3FFFFFFFu))];
-          v[r] = record_key(wd, weight_code<WFMT>(g.w, e, shift) | (d << 16));
+          const uint32_t low = WFMT == 1 ? (uint32_t)(r * 32 + lane) : weight_code<WFMT>(g.w, e, shift);
+          v[r] = ((unsigned long long)d << 48) | ((unsigned long long)(wd & 0x3FFFFFFFu) << 18) |
+                 ((unsigned long long)(wd >> 30) << 16) | (unsigned long long)low;
         }
       }
       warp_bitonic_sort<R>(v, lane);
       int runs = 0;
-      uint32_t last = 0xFFFFFFFFu;  // key of the element before this round's first
+      RunHeads rh;
 #pragma unroll
       for (int r = 0; r < R; r++) {
         const int64_t e = c0 + r * 32 + lane;
         const bool valid = e < r1;
-        const uint2 rec = key_record(v[r]);
-        const uint32_t k = valid ? record_run_key(rec, bins) : 0xFFFFFFFFu;
-        uint32_t left = __shfl_up_sync(0xFFFFFFFFu, k, 1);
-        if (lane == 0) left = last;
-        runs += __popc(__ballot_sync(0xFFFFFFFFu, valid && k != left));
-        last = __shfl_sync(0xFFFFFFFFu, k, 31);
-        if (valid) out[e] = rec;
+        const uint32_t word = (uint32_t)((v[r] >> 18) & 0x3FFFFFFFu) | ((uint32_t)((v[r] >> 16) & 3u) << 30);
+        const uint32_t d = (uint32_t)(v[r] >> 48) & 0xFFu;
+        const uint32_t k = valid ? synapse_run_key(word, d, bins) : 0xFFFFFFFFu;
+        runs += __popc(rh.round(k, valid, r * 32 + lane, lane, !bins));
+        if (valid) {
+          const uint32_t low = (uint32_t)(v[r] & 0xFFFFu);
+          const uint32_t code = WFMT == 1 ? weight_code<1>(g.w, c0 + low, 0) : low;
+          out[e] = make_uint2(word, bins ? code : (uint32_t)decode_weight(code, WFMT, g.wshift));
+          delays[e] = (uint8_t)d;
+        }
       }
       if (lane == 0) counts[chunk] = runs;
     }
@@ -213,10 +227,10 @@ __global__ void __launch_bounds__(256) pack_fill_kernel(DevNet g, uint2* out, in
 
 // Warp per row, after pack_fill and the run pointers: every chunk's run
 // records (key | start << 14 | (length - 1) << 23) at runs[run_ptr[chunk]..],
-// and each packed record's delay byte replaced by its run's index.
-__global__ void __launch_bounds__(256) run_fill_kernel(DevNet g, uint2* pack, const int64_t* run_ptr,
-                                                       uint32_t* runs) {
-  constexpr int R = kItemEvents / 32;
+// in bins mode each packed record's run index above its weight code, and in
+// the queue mode the chunk's info.
+__global__ void __launch_bounds__(256) run_fill_kernel(DevNet g, uint2* pack, const uint8_t* delays,
+                                                       const int64_t* run_ptr, uint32_t* runs, ChunkInfo* info) {
   const int lane = threadIdx.x & 31;
   const bool bins = g.mode == kModeBins;
   const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -225,45 +239,38 @@ __global__ void __launch_bounds__(256) run_fill_kernel(DevNet g, uint2* pack, co
     const int64_t r0 = g.row_ptr[s], r1 = g.row_ptr[s + 1];
     int64_t chunk = g.chunk_base[s];
     for (int64_t c0 = r0; c0 < r1; c0 += kItemEvents, chunk++) {
-      uint32_t k[R];
-      uint2 rec[R];
-#pragma unroll
-      for (int r = 0; r < R; r++) {
-        const int64_t e = c0 + r * 32 + lane;
-        rec[r] = e < r1 ? pack[e] : make_uint2(0u, 0u);
-        k[r] = e < r1 ? record_run_key(rec[r], bins) : 0xFFFFFFFFu;
-      }
+      const int n = (int)min((int64_t)kItemEvents, r1 - c0);
       uint32_t* out = runs + run_ptr[chunk];
+      RunHeads rh;
       int before = 0;  // runs that start before this round
-      bool tail[R];
-      int idx[R];
-#pragma unroll
-      for (int r = 0; r < R; r++) {
-        uint32_t left = __shfl_up_sync(0xFFFFFFFFu, k[r], 1);
-        const uint32_t prev_last = r > 0 ? __shfl_sync(0xFFFFFFFFu, k[r > 0 ? r - 1 : 0], 31) : 0xFFFFFFFFu;
-        if (lane == 0) left = prev_last;
-        uint32_t right = __shfl_down_sync(0xFFFFFFFFu, k[r], 1);
-        const uint32_t next_first = r + 1 < R ? __shfl_sync(0xFFFFFFFFu, k[r + 1 < R ? r + 1 : r], 0) : 0xFFFFFFFFu;
-        if (lane == 31) right = next_first;
-        const bool valid = k[r] != 0xFFFFFFFFu;
-        const bool head = valid && k[r] != left;
-        tail[r] = valid && k[r] != right;
-        const unsigned hb = __ballot_sync(0xFFFFFFFFu, head);
-        idx[r] = before + __popc(hb & (0xFFFFFFFFu >> (31 - lane))) - 1;
-        if (head) out[idx[r]] = k[r] | ((uint32_t)(r * 32 + lane) << 14);
-        before += __popc(hb);
+      int n1 = 0;      // synapses of delay 1
+      for (int p = 0; p < n; p += 32) {
+        const int64_t e = c0 + p + lane;
+        const bool valid = p + lane < n;
+        const uint2 rec = valid ? pack[e] : make_uint2(0u, 0u);
+        const uint32_t k = valid ? synapse_run_key(rec.x, delays[e], bins) : 0xFFFFFFFFu;
+        const unsigned heads = rh.round(k, valid, p + lane, lane, !bins);
+        const int idx = before + __popc(heads & (0xFFFFFFFFu >> (31 - lane))) - 1;
+        if ((heads >> lane) & 1u) out[idx] = k | ((uint32_t)(p + lane) << 14);
+        if (bins && valid) pack[e].y = (rec.y & 0xFFFFu) | ((uint32_t)idx << 16);
+        before += __popc(heads);
+        n1 += __popc(__ballot_sync(0xFFFFFFFFu, valid && (k & kRunRegion)));
       }
+      if (info && lane == 0) info[chunk] = chunk_info(c0, n, n1, run_ptr[chunk], before);
       __syncwarp();
-#pragma unroll
-      for (int r = 0; r < R; r++) {
-        const int64_t e = c0 + r * 32 + lane;
-        if (tail[r]) {
-          const uint32_t h = out[idx[r]];
-          out[idx[r]] = h | ((uint32_t)(r * 32 + lane - run_start(h)) << 23);
+      // lengths: up to the next run's start
+      for (int r0_ = 0; r0_ < before; r0_ += 32) {
+        const int r = r0_ + lane;
+        uint32_t mine = 0;
+        int next = n;
+        if (r < before) {
+          mine = out[r];
+          if (r + 1 < before) next = run_start(out[r + 1]);
         }
-        if (e < r1) pack[e] = make_uint2(rec[r].x, (rec[r].y & 0xFFFFu) | ((uint32_t)idx[r] << 16));
+        __syncwarp();
+        if (r < before) out[r] = mine | ((uint32_t)(next - run_start(mine) - 1) << 23);
+        __syncwarp();
       }
-      __syncwarp();
     }
   }
 }
@@ -298,79 +305,70 @@ __global__ void ring_gather_kernel(DevNet g, const int64_t* idx, int64_t m, int3
   out[k] = g.ring[sc * g.npad + idx[r]];
 }
 
-// ---- event-queue mode: the dense ring view of the pending events ----
-// Queue x (x != t mod D) holds the events arriving at the step congruent to x;
-// the one-slot accumulator holds slot t mod D (t = the next step to run).
-// Bins mode: every queue is a slot (x_acc = -1) and its events carry weight
-// codes.
-__device__ __forceinline__ int32_t queued_weight(const DevNet& g, uint32_t w) {
-  return g.mode == kModeBins ? decode_weight(w, g.wfmt, g.wshift) : (int32_t)w;
-}
-
-// Test hook of the counters: every queue (blockIdx.y < D) and, in bins mode,
-// every bin (blockIdx.y = D + parity * n_reg + region) gets its unused
-// entries filled with placeholder events of weight 0 (target 0, class 0,
-// weight code 0), then its count set to value (>= its capacity).
+// ---- queue and bins modes: the dense ring view of the pending events ----
+// Queue x holds what arrives at the step congruent to x: runs of synapses in the
+// queue mode, events in bins mode.  In the queue mode slot t mod D (t = the next
+// step to run) is the accumulator's and its queue is drained (x_acc; -1 in bins
+// mode).
+// Test hook of the counters: every queue (blockIdx.y < nq = D * n_sub) and, in
+// bins mode, every bin (blockIdx.y = nq + parity * n_reg + region) gets its unused
+// entries filled with placeholders of weight 0 (target 0, class 0, weight code
+// 0; a queued run is the one record past the last synapse), then its count set
+// to value (>= its capacity).
 __global__ void preset_counters_kernel(DevNet g, unsigned long long value) {
-  const int64_t y = blockIdx.y;
-  const bool queue = y < g.D;
+  const int64_t y = blockIdx.y, nq = (int64_t)g.D * g.n_sub;
+  const bool queue = y < nq;
   const int64_t cap = queue ? g.qcap : g.bcap;
-  unsigned long long* cnt = queue ? g.qcnt + y * kQcntStride : g.bcnt + (y - g.D) * kBcntStride;
+  unsigned long long* cnt = queue ? g.qcnt + y * kQcntStride : g.bcnt + (y - nq) * kBcntStride;
   const int64_t used = (int64_t)min(*cnt, (unsigned long long)cap);
   for (int64_t i = used + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cap; i += (int64_t)gridDim.x * blockDim.x) {
-    if (queue) g.q[y * g.qcap + i] = make_uint2(0u, 0u);
-    else if (g.ev8) reinterpret_cast<uint2*>(g.bins)[(y - g.D) * g.bcap + i] = make_uint2(0u, 0u);
-    else g.bins[(y - g.D) * g.bcap + i] = 0u;
+    if (queue) g.q[y * g.qcap + i] = g.mode == kModeBins ? 0ull : run_desc(g.nnz, 1);
+    else if (g.ev8) reinterpret_cast<uint2*>(g.bins)[(y - nq) * g.bcap + i] = make_uint2(0u, 0u);
+    else g.bins[(y - nq) * g.bcap + i] = 0u;
   }
 }
 
 __global__ void set_counters_kernel(DevNet g, unsigned long long value) {
   const int64_t y = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t nb = g.mode == kModeBins ? 2 * (int64_t)g.n_reg : 0;
-  if (y < g.D) g.qcnt[y * kQcntStride] = value;
-  else if (y < g.D + nb) g.bcnt[(y - g.D) * kBcntStride] = value;
+  const int64_t nq = (int64_t)g.D * g.n_sub;
+  if (y < nq) g.qcnt[y * kQcntStride] = value;
+  else if (y < nq + nb) g.bcnt[(y - nq) * kBcntStride] = value;
+}
+
+// Every pending event of step x's queues: f(class, target, weight).
+template <typename F>
+__device__ __forceinline__ void for_queued(const DevNet& g, int32_t x, F&& f) {
+  const bool bins = g.mode == kModeBins;
+  for (int64_t s = (int64_t)x * g.n_sub; s < (int64_t)(x + 1) * g.n_sub; s++) {
+    const int64_t cnt = (int64_t)min(g.qcnt[s * kQcntStride], (unsigned long long)g.qcap);
+    const unsigned long long* q = g.q + s * g.qcap;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (int64_t)gridDim.x * blockDim.x) {
+      if (bins) {
+        const uint2 e = reinterpret_cast<const uint2*>(q)[i];
+        f(e.x >> 30, e.x & 0x3FFFFFFFu, decode_weight(e.y, g.wfmt, g.wshift));
+      } else {
+        const uint2* rec = g.syn_pack + desc_first(q[i]);
+        const int len = desc_len(q[i]);
+        for (int k = 0; k < len; k++) f(rec[k].x >> 30, rec[k].x & 0x3FFFFFFFu, (int32_t)rec[k].y);
+      }
+    }
+  }
 }
 
 __global__ void queue_to_dense_kernel(DevNet g, int32_t* dense, int32_t x_acc) {
   const int32_t x = blockIdx.y;
   if (x == x_acc) return;
-  const int64_t cnt = (int64_t)min(g.qcnt[x * kQcntStride], (unsigned long long)g.qcap);
-  const uint2* q = g.q + (int64_t)x * g.qcap;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (int64_t)gridDim.x * blockDim.x) {
-    const uint2 e = q[i];
-    atomicAdd(dense + ((int64_t)x * g.nch + (e.x >> 30)) * g.npad + (e.x & 0x3FFFFFFFu), queued_weight(g, e.y));
-  }
-}
-
-__global__ void dense_to_queue_kernel(DevNet g, const int32_t* dense, int32_t x_acc) {
-  const int32_t x = blockIdx.y;
-  if (x == x_acc) return;
-  const int64_t per = (int64_t)g.nch * g.npad;
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < per; k += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t c = (int32_t)(k / g.npad);
-    const int64_t i = k - (int64_t)c * g.npad;
-    const int32_t w = dense[(int64_t)x * per + k];
-    if (w == 0 || i >= g.n) continue;
-    const unsigned long long pos = atomicAdd(g.qcnt + x * kQcntStride, 1ull);
-    if (pos >= (unsigned long long)g.qcap) {
-      atomicAdd(g.spill + (int64_t)x * per + k, w);
-      g.spill_dirty[x] = 1;
-      continue;
-    }
-    g.q[(int64_t)x * g.qcap + pos] = make_uint2((uint32_t)i | ((uint32_t)c << 30), (uint32_t)w);
-  }
+  for_queued(g, x, [&](uint32_t c, uint32_t tgt, int32_t w) {
+    atomicAdd(dense + ((int64_t)x * g.nch + c) * g.npad + tgt, w);
+  });
 }
 
 __global__ void queue_sums_kernel(DevNet g, unsigned long long* sums, int32_t x_acc) {
   const int32_t x = blockIdx.y;
   if (x == x_acc) return;
-  const int64_t cnt = (int64_t)min(g.qcnt[x * kQcntStride], (unsigned long long)g.qcap);
-  const uint2* q = g.q + (int64_t)x * g.qcap;
   long long acc[4] = {0, 0, 0, 0};
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (int64_t)gridDim.x * blockDim.x) {
-    const uint2 e = q[i];
-    acc[e.x >> 30] += queued_weight(g, e.y);
-  }
+  for_queued(g, x, [&](uint32_t c, uint32_t, int32_t w) { acc[c] += w; });
   for (int c = 0; c < 4; c++) {
     long long a = acc[c];
     for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xFFFFFFFFu, a, o);
@@ -382,13 +380,10 @@ __global__ void queue_sums_kernel(DevNet g, unsigned long long* sums, int32_t x_
 __global__ void queue_gather_kernel(DevNet g, const int32_t* map, int32_t* out, int32_t x_acc) {
   const int32_t x = blockIdx.y;
   if (x == x_acc) return;
-  const int64_t cnt = (int64_t)min(g.qcnt[x * kQcntStride], (unsigned long long)g.qcap);
-  const uint2* q = g.q + (int64_t)x * g.qcap;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (int64_t)gridDim.x * blockDim.x) {
-    const uint2 e = q[i];
-    const int32_t r = map[e.x & 0x3FFFFFFFu];
-    if (r >= 0) atomicAdd(out + ((int64_t)r * g.D + x) * g.nch + (e.x >> 30), queued_weight(g, e.y));
-  }
+  for_queued(g, x, [&](uint32_t c, uint32_t tgt, int32_t w) {
+    const int32_t r = map[tgt];
+    if (r >= 0) atomicAdd(out + ((int64_t)r * g.D + x) * g.nch + c, w);
+  });
 }
 
 // Bins mode: between calls the bins of parity x mod 2 hold the delay-1 events
@@ -517,16 +512,11 @@ cudaError_t launch_add(int32_t* dst, const int32_t* src, int64_t n, cudaStream_t
 }
 
 cudaError_t launch_preset_counters(const DevNet& g, unsigned long long value, cudaStream_t st) {
-  const int64_t rows = g.D + (g.mode == kModeBins ? 2 * (int64_t)g.n_reg : 0);
+  const int64_t rows = (int64_t)g.D * g.n_sub + (g.mode == kModeBins ? 2 * (int64_t)g.n_reg : 0);
   preset_counters_kernel<<<dim3(8, (unsigned)rows), 256, 0, st>>>(g, value);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   set_counters_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(g, value);  // after every fill has read its count
-  return cudaGetLastError();
-}
-
-cudaError_t launch_dense_to_queue(const DevNet& g, const int32_t* dense, int32_t x_acc, cudaStream_t st) {
-  dense_to_queue_kernel<<<dim3(64, (unsigned)g.D), 256, 0, st>>>(g, dense, x_acc);
   return cudaGetLastError();
 }
 
@@ -583,24 +573,25 @@ cudaError_t launch_delay_fill(const DevNet& g, uint8_t* out, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_pack_fill(const DevNet& g, uint2* out, int32_t* counts, cudaStream_t st) {
+cudaError_t launch_pack_fill(const DevNet& g, uint2* out, uint8_t* delays, int32_t* counts, cudaStream_t st) {
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   switch (g.wfmt) {
-    case 0: pack_fill_kernel<0><<<sms * 8, 256, 0, st>>>(g, out, counts); break;
-    case 2: pack_fill_kernel<2><<<sms * 8, 256, 0, st>>>(g, out, counts); break;
-    case 3: pack_fill_kernel<3><<<sms * 8, 256, 0, st>>>(g, out, counts); break;
-    default: return cudaErrorInvalidValue;  // int32 weights do not fit a 16-bit code
+    case 0: pack_fill_kernel<0><<<sms * 8, 256, 0, st>>>(g, out, delays, counts); break;
+    case 1: pack_fill_kernel<1><<<sms * 8, 256, 0, st>>>(g, out, delays, counts); break;
+    case 2: pack_fill_kernel<2><<<sms * 8, 256, 0, st>>>(g, out, delays, counts); break;
+    default: pack_fill_kernel<3><<<sms * 8, 256, 0, st>>>(g, out, delays, counts); break;
   }
   return cudaGetLastError();
 }
 
-cudaError_t launch_run_fill(const DevNet& g, uint2* pack, const int64_t* run_ptr, uint32_t* runs, cudaStream_t st) {
+cudaError_t launch_run_fill(const DevNet& g, uint2* pack, const uint8_t* delays, const int64_t* run_ptr,
+                            uint32_t* runs, ChunkInfo* info, cudaStream_t st) {
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  run_fill_kernel<<<sms * 8, 256, 0, st>>>(g, pack, run_ptr, runs);
+  run_fill_kernel<<<sms * 8, 256, 0, st>>>(g, pack, delays, run_ptr, runs, info);
   return cudaGetLastError();
 }
 
