@@ -100,7 +100,9 @@ enum {
 
 /* How delivered events wait out their delay (the results are the same bit for bit;
  * DTB_DELIVER_BINS without a bin_capacity of the caller's keeps the queue layout
- * for networks whose accumulators are at most 24 MiB: it is the faster one there). */
+ * for networks whose accumulators are at most 24 MiB, and both keep the ring, without
+ * capacities of the caller's, for networks of at most 3,072 neurons with at most 200
+ * synapses per neuron: they are the faster ones there). */
 enum {
   DTB_DELIVER_RING = 0,  /* dense ring acc[D][n_channels][N]: every synapse event is one int32
                             reduction into slot (t + d) mod D */

@@ -43,6 +43,15 @@ dtb_status cuda_fail(cudaError_t e, const char* where) {
   } while (0)
 
 constexpr int kGraphSteps = 32;
+constexpr int64_t kSmallSteps = 4096;  // steps per launch of a small network (some ten milliseconds)
+// Synapses per neuron up to which a small network's steps run in one CTA: its
+// warps take one spike's row each, so a step takes longer the longer the rows
+// and the more spikes.  3,000 neurons at 8 Hz, us per step of the launches and of
+// the one CTA: 7.6 and 4.3 with 150 synapses per neuron, 7.7 and 4.7 with 200,
+// 7.8 and 5.9 with 300 (in 40 voxels 8.7 and 9.5), 8.6 and 13.5 with 1,000.
+// At 150 the two meet near 100 Hz; 1,000 neurons: 6.8 and 3.3 at 10 Hz, 9.5 and
+// 7.9 at 117 Hz.
+constexpr int64_t kSmallInDegree = 200;
 constexpr int kTimedKernels = 5;  // update, compaction, delivery, drain or binning, BOLD
 // Networks of at most this many 1,024-neuron blocks run the compaction of a
 // step beside the neuron update of the next by default: their kernels leave
@@ -84,6 +93,8 @@ struct dtb_net {
   int update_stages = 3;     // neuron update pipeline depth
   int update_per_sm = 0;     // neuron update CTAs per SM (0 = as many as fit)
   int schedule = -1;         // requested: -1 by size, 0 compaction after the update, 1 beside the next update
+  bool small = false;        // a call's steps run in one CTA (launch_small_steps)
+  bool routed = false;       // the layout in use is not the one asked for
   bool beside = false;       // in effect: the compaction of step t runs beside the update of step t + 1
   // the second copy of the spike bits (words) and of the block counts (blocks)
   int64_t flag_par = 0;
@@ -423,6 +434,11 @@ dtb_status enqueue_tail(dtb_net* net) {
 
 // A whole call of n >= 1 steps, the body in graph chunks when it is long.
 dtb_status enqueue_call(dtb_net* net, int64_t n, bool use_graph) {
+  if (net->small) {
+    for (int64_t left = n; left > 0; left -= kSmallSteps)
+      DTB_CUDA(dtb::launch_small_steps(net->g, (int32_t)std::min(left, kSmallSteps), net->stream));
+    return DTB_OK;
+  }
   dtb_status s = enqueue_range(net, 1, true);
   if (s != DTB_OK) return s;
   int64_t left = n - 1;
@@ -462,7 +478,7 @@ dtb_status build_graph(dtb_net* net, int32_t k) {
 // The graphs a call of n steps launches (full chunks and the remainder), built
 // before any of its work is queued.
 dtb_status ensure_graphs(dtb_net* net, int64_t n) {
-  if (n < 2) return DTB_OK;
+  if (n < 2 || net->small) return DTB_OK;
   const int64_t body = n - 1;
   const int32_t rem = (int32_t)(body % kGraphSteps);
   if (body >= kGraphSteps && !net->graph[kGraphSteps]) {
@@ -666,9 +682,31 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
   g.bold_cap = kBoldLogCap;
   g.log_cap = d->spike_log_capacity > 0 ? d->spike_log_capacity : ((int64_t)1 << 25);
   g.mode = d->delivery_mode;
+  int64_t nnz = 0;
+  if (d->csr_on_device) {
+    const cudaError_t e = cudaMemcpy(&nnz, d->row_ptr + n, 8, cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) {
+      delete net;
+      return cuda_fail(e, "reading row_ptr[n]");
+    }
+  } else {
+    nnz = d->row_ptr[n];
+  }
+  // layouts without capacities of the caller's: the ring for the smallest
+  // networks (whose steps run in one CTA), the queues where the accumulator fits
+  // the cache
+  const bool free_layout = d->bin_capacity == 0 && d->event_queue_capacity == 0;
+  const bool few = dtb::small_network(g) && nnz <= kSmallInDegree * n;
+  if (g.mode && free_layout && few) {
+    g.mode = dtb::kModeRing;
+    net->routed = true;
+  }
   if (g.mode == dtb::kModeBins && n <= (int64_t)dtb::kMaxRegions * dtb::kRegionNeurons && d->bin_capacity == 0 &&
-      4 * npad * g.nch <= kQueueMaxBytes)
+      4 * npad * g.nch <= kQueueMaxBytes) {
     g.mode = dtb::kModeQueue;
+    net->routed = true;
+  }
+  net->small = g.mode == dtb::kModeRing && few;
   g.ou = d->ou_enable ? 1 : 0;
   net->ou_mu = d->ou_mu;
   if (g.ou) {
@@ -787,19 +825,12 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
   }
 
   // synapses: adopt device arrays or copy host arrays
-  int64_t nnz = 0;
   if (d->csr_on_device) {
-    e = cudaMemcpy(&nnz, d->row_ptr + n, 8, cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) {
-      delete net;
-      return cuda_fail(e, "reading row_ptr[n]");
-    }
     g.row_ptr = d->row_ptr;
     g.word = d->syn_word;
     g.w = d->syn_w;
     g.row_shift = d->row_shift;
   } else {
-    nnz = d->row_ptr[n];
     if (d->row_ptr[0] != 0 || nnz < 0) {
       delete net;
       return fail(DTB_EINVAL, "row_ptr must start at 0 and end at nnz >= 0");
@@ -1737,9 +1768,10 @@ dtb_status dtb_spike_compact(const uint32_t* d_bits, int64_t n, int32_t* d_ids, 
 
 dtb_status dtb_test_preset_counters(dtb_net* net, uint64_t value) {
   if (!net) return fail(DTB_EINVAL, "net is NULL");
-  if (net->g.mode == dtb::kModeRing) return fail(DTB_ESTATE, "the ring mode keeps no event queues");
+  if (net->g.mode == dtb::kModeRing && !net->routed) return fail(DTB_ESTATE, "the ring mode keeps no event queues");
   const uint64_t cap = (uint64_t)std::max<int64_t>(net->g.qcap, net->g.mode == dtb::kModeBins ? net->g.bcap : 0);
   if (value < cap || value > ((uint64_t)1 << 62)) return fail(DTB_EINVAL, "value out of capacity .. 2^62");
+  if (net->g.mode == dtb::kModeRing) return DTB_OK;  // a layout without counters was chosen
   DTB_CUDA(dtb::launch_preset_counters(net->g, (unsigned long long)value, net->stream));
   DTB_CUDA(cudaStreamSynchronize(net->stream));
   return DTB_OK;

@@ -24,6 +24,10 @@ cudaError_t launch_bin(const DevNet& g, int32_t t_rel, cudaStream_t st);
 cudaError_t launch_bold_step(const DevNet& g, int32_t t_rel, cudaStream_t st);
 cudaError_t launch_advance(const DevNet& g, int32_t k, cudaStream_t st);
 cudaError_t launch_begin_call(const DevNet& g, cudaStream_t st);
+// Networks of a few blocks in ring mode: n_steps whole steps in one CTA (the
+// step counter moves on, the spike log grows).
+bool small_network(const DevNet& g);
+cudaError_t launch_small_steps(const DevNet& g, int32_t n_steps, cudaStream_t st);
 int deliver_blocks_per_sm();
 // Attributes of the step's kernels on the current device (once per network).
 cudaError_t prepare_step_kernels();

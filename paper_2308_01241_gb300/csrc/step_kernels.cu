@@ -927,6 +927,21 @@ __device__ __forceinline__ int lower_bound(const int32_t* a, int n, int32_t x) {
   return lo;
 }
 
+// Balloon-Windkessel, one Euler step of one voxel's state s, f, v, q at input z (Hz).
+__device__ __forceinline__ float bold_euler(const BoldConst& b, float z, float& s, float& f, float& vv, float& q) {
+  const float fout = powf(vv, b.inv_alpha);
+  const float Ef = 1.0f - expf(b.ln_1mE0 / f);
+  const float ds = b.eps * z - s * b.inv_tau_s - (f - 1.0f) * b.inv_tau_f;
+  const float df = s;
+  const float dv = (f - fout) * b.inv_tau_0;
+  const float dq = (f * Ef * b.inv_E0 - fout * q / vv) * b.inv_tau_0;
+  s += b.dt_s * ds;
+  f += b.dt_s * df;
+  vv += b.dt_s * dv;
+  q += b.dt_s * dq;
+  return b.V0 * (b.k1 * (1.0f - q) + b.k2 * (1.0f - q / vv) + b.k3 * (1.0f - vv));
+}
+
 // Balloon-Windkessel, one thread per voxel.  z = spikes / (n_v * dt) in Hz,
 // counted by binary search of the voxel's id range in the ascending list.
 __global__ void bold_step_kernel(DevNet g, int32_t t_rel) {
@@ -938,20 +953,9 @@ __global__ void bold_step_kernel(DevNet g, int32_t t_rel) {
   const int cnt = lower_bound(spk, n_spk, g.vstart[v + 1]) - lower_bound(spk, n_spk, g.vstart[v]);
   g.vox_spikes[v] += (unsigned long long)cnt;
   const float z = (float)cnt * g.inv_nvox[v];
-  const BoldConst& b = g.bc;
   const int nv = g.nv;
   float s = g.bold[v], f = g.bold[nv + v], vv = g.bold[2 * nv + v], q = g.bold[3 * nv + v];
-  const float fout = powf(vv, b.inv_alpha);
-  const float Ef = 1.0f - expf(b.ln_1mE0 / f);
-  const float ds = b.eps * z - s * b.inv_tau_s - (f - 1.0f) * b.inv_tau_f;
-  const float df = s;
-  const float dv = (f - fout) * b.inv_tau_0;
-  const float dq = (f * Ef * b.inv_E0 - fout * q / vv) * b.inv_tau_0;
-  s += b.dt_s * ds;
-  f += b.dt_s * df;
-  vv += b.dt_s * dv;
-  q += b.dt_s * dq;
-  const float y = b.V0 * (b.k1 * (1.0f - q) + b.k2 * (1.0f - q / vv) + b.k3 * (1.0f - vv));
+  const float y = bold_euler(g.bc, z, s, f, vv, q);
   g.bold[v] = s;
   g.bold[nv + v] = f;
   g.bold[2 * nv + v] = vv;
@@ -960,6 +964,256 @@ __global__ void bold_step_kernel(DevNet g, int32_t t_rel) {
   if (g.bold_every > 0 && (t + 1) % g.bold_every == 0) {
     const int64_t idx = (t + 1) / g.bold_every - 1;
     g.bold_log[(idx % g.bold_cap) * nv + v] = y;
+  }
+}
+
+// ---- networks of at most kSmallBlocks blocks: a call in one CTA ----
+//
+// A step of a network of a few thousand neurons is a chain of dependent
+// launches: 6.9 us a step for 1,000 neurons with 100 synapses each, whose
+// arithmetic takes well under one (2.8 us with this kernel).  Here one CTA runs
+// all the steps of a call with V, j and the refractory counters in registers
+// (four neurons per thread); only the delay ring, the synapses and the BOLD state
+// are in global memory.  One barrier a step:
+//   before it  j part of step t - 1 and V part of step t; the spikes go to a
+//              list in shared memory with their rows' bounds;
+//   barrier    the list is complete, and what step t - 1 delivered is visible;
+//   after it   the arrivals of step t are fetched for the next iteration (they
+//              were all delivered by step t - 1) and the list's rows are
+//              delivered, a warp each; helper warps without neurons advance the
+//              spike log and the BOLD step as well.
+// What bounds a step is the chain of one trip to L2 for the rows, one for the
+// sums, and the neuron's own arithmetic.
+constexpr int kSmallBlocks = 3;
+
+__device__ __forceinline__ int32_t synapse_weight(const DevNet& g, int64_t e, int32_t src) {
+  switch (g.wfmt) {
+    case 0: return decode_weight(weight_code<0>(g.w, e, 0), 0, g.wshift);
+    case 1: return decode_weight(weight_code<1>(g.w, e, 0), 1, g.wshift);
+    case 2: return decode_weight(weight_code<2>(g.w, e, 0), 2, g.wshift);
+    default: return decode_weight(weight_code<3>(g.w, e, g.wshift + (g.row_shift ? g.row_shift[src] : 0)), 3, g.wshift);
+  }
+}
+
+// Dynamic shared memory: spike list and rows, two copies (a list is read after
+// its step's barrier and written again before the barrier two steps on); counts,
+// bits and voxel counts [nv], three copies (step k clears those of step k + 2,
+// which nobody touches between the barriers around it).
+struct SmallSmem {
+  static constexpr int kN = kSmallBlocks * kNeuronsPerBlock;
+  static constexpr size_t kRow = 0;                          // int64 [2][kN] row starts
+  static constexpr size_t kLen = kRow + 2 * kN * 8;          // int32 [2][kN] row lengths
+  static constexpr size_t kId = kLen + 2 * kN * 4;           // int32 [2][kN] ids, in no order
+  static constexpr size_t kBits = kId + 2 * kN * 4;          // uint32 [3][kN / 32]
+  static constexpr size_t kVox = kBits + 3 * (kN / 32) * 4;  // int32 [3][nv]
+  static constexpr size_t bytes(int nv) { return kVox + 3 * (size_t)nv * 4; }
+};
+
+template <int NCH, bool OU, int MAXT>
+__global__ void __launch_bounds__(MAXT, 1) small_steps_kernel(DevNet g, int32_t n_steps) {
+  using L = SmallSmem;
+  extern __shared__ __align__(16) unsigned char ssm[];
+  int64_t* s_row = reinterpret_cast<int64_t*>(ssm + L::kRow);
+  int32_t* s_len = reinterpret_cast<int32_t*>(ssm + L::kLen);
+  int32_t* s_id = reinterpret_cast<int32_t*>(ssm + L::kId);
+  uint32_t* s_bits = reinterpret_cast<uint32_t*>(ssm + L::kBits);
+  int32_t* s_vox = reinterpret_cast<int32_t*>(ssm + L::kVox);
+  __shared__ int s_n[3];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nthr = g.nblk * kUpdateThreads, nwarp = nthr / 32;  // with neurons
+  const int nhelp = (int)blockDim.x - nthr;                      // threads without
+  const bool helper = tid >= nthr;
+  const int nv = g.nv;
+  const int64_t np = g.npad, t0 = *g.t_base;
+  const int64_t i0 = (int64_t)tid * 4;
+  // my neurons
+  Quad s = {};
+  if (!helper) {
+    const float4 v = *reinterpret_cast<const float4*>(g.V + i0);
+    s.V[0] = v.x; s.V[1] = v.y; s.V[2] = v.z; s.V[3] = v.w;
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      const float4 j = *reinterpret_cast<const float4*>(g.j + q * np + i0);
+      s.J[q][0] = j.x; s.J[q][1] = j.y; s.J[q][2] = j.z; s.J[q][3] = j.w;
+    }
+    s.ref4 = *reinterpret_cast<const uint32_t*>(g.ref + i0);
+    const float4 I = OU ? *reinterpret_cast<const float4*>(g.Iou + i0) : make_float4(0.f, 0.f, 0.f, 0.f);
+    s.I[0] = I.x; s.I[1] = I.y; s.I[2] = I.z; s.I[3] = I.w;
+  }
+  int32_t v0 = 0;  // voxel of my first neuron
+  while (!helper && v0 + 1 < nv && g.vstart[v0 + 1] <= i0) v0++;
+  const bool mixed = v0 + 1 < nv && g.vstart[v0 + 1] <= i0 + 3;
+  // BOLD: a helper's first voxel (from the last thread on) in registers, further
+  // ones through memory
+  const int my_vox = helper ? (int)blockDim.x - 1 - tid : nv;
+  float bs = 0.f, bf = 1.f, bv = 1.f, bq = 1.f, by = 0.f;
+  unsigned long long vox_total = 0;
+  if (my_vox < nv) {
+    bs = g.bold[my_vox]; bf = g.bold[nv + my_vox]; bv = g.bold[2 * nv + my_vox]; bq = g.bold[3 * nv + my_vox];
+    by = g.bold[4 * nv + my_vox];
+  }
+  int64_t log_pos = g.log_pos[t0 & 1];
+  const int32_t cs0 = *g.call_steps;
+  bool trunc = false;
+  unsigned long long events = 0, spikes = 0;
+  for (int k = tid; k < 3 * nv; k += (int)blockDim.x) s_vox[k] = 0;
+  for (int k = tid; k < 3 * L::kN / 32; k += (int)blockDim.x) s_bits[k] = 0;
+  if (tid < 3) s_n[tid] = 0;
+  __syncthreads();
+
+  int32_t slot = (int32_t)(t0 % g.D);  // of step t
+  int4 A4[NCH];                        // arrivals of the step before
+#pragma unroll
+  for (int cc = 0; cc < NCH; cc++) A4[cc] = make_int4(0, 0, 0, 0);
+  bool sent = false;                   // this warp delivered in the step before
+  auto j_part = [&](int64_t x) {
+    const uint4 r = philox4x32_10(make_uint4((uint32_t)(i0 >> 2), (uint32_t)x, (uint32_t)((uint64_t)x >> 32), kTagDrive),
+                                  g.key0, g.key1);
+    const uint32_t u[4] = {r.x, r.y, r.z, r.w};
+    int32_t kp[4];
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      kp[q] = poisson_low(g, u[q]);
+      if (g.M > 3 && u[q] >= g.T[2]) kp[q] += poisson_high(g, u[q]);
+    }
+    if (!mixed) quad_j<NCH>(g, g.vc[v0], s, A4, kp);
+    else (void)quad_mixed<NCH, false>(g, s, A4, kp, i0, x, v0, false, true, false);
+  };
+  auto fetch = [&](int32_t sl) {  // my neurons' sums of slot sl, which are cleared
+#pragma unroll
+    for (int cc = 0; cc < NCH; cc++) {
+      int4* p = reinterpret_cast<int4*>(g.ring + ((int64_t)sl * NCH + cc) * np + i0);
+      A4[cc] = __ldcg(p);
+      if (A4[cc].x | A4[cc].y | A4[cc].z | A4[cc].w) __stcg(p, make_int4(0, 0, 0, 0));
+    }
+  };
+  for (int32_t k = 0, c = 0; k < n_steps; k++, c = c == 2 ? 0 : c + 1) {  // c: copy k mod 3
+    const int64_t t = t0 + k;
+    const int par = k & 1;
+    uint32_t* bits = s_bits + c * (L::kN / 32);
+    int32_t* vox = s_vox + c * nv;
+    if (k > 0 && !helper) j_part(t - 1);
+    uint32_t nib = 0;
+    if (helper) {
+    } else if (!mixed) {
+      nib = quad_v<OU>(g, g.vc[v0], s, i0, t);
+    } else {
+      const int32_t none[4] = {0, 0, 0, 0};
+      nib = quad_mixed<NCH, OU>(g, s, A4, none, i0, t, v0, true, false, false);
+    }
+    if (i0 + 3 >= g.n) nib &= i0 >= g.n ? 0u : (1u << (g.n - i0)) - 1u;  // padding never fires
+    if (nib) {
+      atomicOr(&bits[tid >> 3], nib << (4 * (tid & 7)));
+      int at = atomicAdd(&s_n[c], __popc(nib));
+#pragma unroll
+      for (int q = 0; q < 4; q++)
+        if ((nib >> q) & 1u) {
+          const int32_t id = (int32_t)i0 + q;
+          const int64_t a = __ldg(g.row_ptr + id);
+          s_id[par * L::kN + at] = id;
+          s_row[par * L::kN + at] = a;
+          s_len[par * L::kN + at] = (int32_t)(__ldg(g.row_ptr + id + 1) - a);
+          int32_t v = v0;
+          while (v + 1 < nv && g.vstart[v + 1] <= id) v++;
+          atomicAdd(&vox[v], 1);
+          at++;
+        }
+    }
+    if (sent) __threadfence();  // my deliveries of step t - 1 before the barrier
+    __syncthreads();
+    const int n = s_n[c];
+    sent = warp < n;
+    if (!helper) fetch(slot);
+    // rows of the list, a warp each (long ones are walked by their warp)
+    for (int l = warp; l < n; l += (int)(blockDim.x >> 5)) {
+      const int64_t a = s_row[par * L::kN + l];
+      const int len = s_len[par * L::kN + l];
+      const int32_t src = s_id[par * L::kN + l];
+      if (lane == 0) events += (unsigned long long)len;
+      for (int e0 = lane; e0 < len; e0 += 128) {
+        uint32_t wd[4];
+        int32_t wa[4], dd[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+          const bool in = e0 + 32 * u < len;
+          const int64_t e = a + (in ? e0 + 32 * u : 0);
+          wd[u] = __ldg(g.word + e);
+          wa[u] = synapse_weight(g, e, src);
+          dd[u] = in ? (int32_t)__ldg(g.syn_delay + e) : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+          if (dd[u] == 0) continue;
+          int32_t sl = slot + dd[u];
+          if (sl >= g.D) sl -= g.D;
+          atomicAdd(g.ring + ((int64_t)sl * NCH + (wd[u] >> 30)) * np + (wd[u] & 0x3FFFFFFFu), wa[u]);
+        }
+      }
+    }
+    // the spike log: a spike's rank is the number of bits below its own
+    if (warp == nwarp) {
+      for (int l = lane; l < n; l += 32) {
+        const int32_t id = s_id[par * L::kN + l];
+        int rank = __popc(bits[id >> 5] & ((1u << (id & 31)) - 1u));
+        for (int w = 0; w < (id >> 5); w++) rank += __popc(bits[w]);
+        if (log_pos + rank < g.log_cap) g.log_ids[log_pos + rank] = id;
+      }
+      log_pos += n;
+      if (log_pos > g.log_cap) {
+        log_pos = g.log_cap;
+        trunc = true;
+      }
+      if (lane == 0) g.step_off[cs0 + k + 1] = log_pos;
+      spikes += (unsigned long long)n;
+    }
+    // BOLD
+    const bool sample = g.bold_every > 0 && (t + 1) % g.bold_every == 0;
+    float* row = sample ? g.bold_log + (((t + 1) / g.bold_every - 1) % g.bold_cap) * nv : nullptr;
+    if (my_vox < nv) {
+      const int fired = vox[my_vox];
+      vox_total += (unsigned long long)fired;
+      by = bold_euler(g.bc, (float)fired * g.inv_nvox[my_vox], bs, bf, bv, bq);
+      if (row) row[my_vox] = by;
+    }
+    for (int v = my_vox + nhelp; v < nv; v += nhelp) {
+      const int fired = vox[v];
+      g.vox_spikes[v] += (unsigned long long)fired;
+      float a = g.bold[v], b = g.bold[nv + v], d = g.bold[2 * nv + v], q = g.bold[3 * nv + v];
+      const float y = bold_euler(g.bc, (float)fired * g.inv_nvox[v], a, b, d, q);
+      g.bold[v] = a; g.bold[nv + v] = b; g.bold[2 * nv + v] = d; g.bold[3 * nv + v] = q; g.bold[4 * nv + v] = y;
+      if (row) row[v] = y;
+    }
+    // clear the copies of step k + 2
+    const int c2 = c == 0 ? 2 : c - 1;
+    if (helper) {
+      if (tid == nthr) s_n[c2] = 0;
+      for (int w = tid - nthr; w < L::kN / 32; w += nhelp) s_bits[c2 * (L::kN / 32) + w] = 0;
+      for (int v = tid - nthr; v < nv; v += nhelp) s_vox[c2 * nv + v] = 0;
+    }
+    slot = slot + 1 == g.D ? 0 : slot + 1;
+  }
+  if (!helper) {
+    j_part(t0 + n_steps - 1);
+    // the state back
+    *reinterpret_cast<float4*>(g.V + i0) = make_float4(s.V[0], s.V[1], s.V[2], s.V[3]);
+#pragma unroll
+    for (int q = 0; q < 4; q++)
+      *reinterpret_cast<float4*>(g.j + q * np + i0) = make_float4(s.J[q][0], s.J[q][1], s.J[q][2], s.J[q][3]);
+    *reinterpret_cast<uint32_t*>(g.ref + i0) = s.ref4;
+    if (OU) *reinterpret_cast<float4*>(g.Iou + i0) = make_float4(s.I[0], s.I[1], s.I[2], s.I[3]);
+  }
+  if (my_vox < nv) {
+    g.bold[my_vox] = bs; g.bold[nv + my_vox] = bf; g.bold[2 * nv + my_vox] = bv; g.bold[3 * nv + my_vox] = bq;
+    g.bold[4 * nv + my_vox] = by;
+    g.vox_spikes[my_vox] += vox_total;
+  }
+  if (lane == 0 && events) atomicAdd(g.events, events);
+  if (tid == nthr) {
+    g.log_pos[0] = g.log_pos[1] = log_pos;
+    if (trunc) *g.log_trunc = 1;
+    *g.call_steps = cs0 + n_steps;
+    *g.spikes += spikes;
+    *g.t_base = t0 + n_steps;
   }
 }
 
@@ -1034,6 +1288,37 @@ cudaError_t launch_neuron_update(const DevNet& g, int32_t t_rel, cudaStream_t st
                 : launch_update_ou<false, true>(g, t_rel, st, stages, blocks_per_sm, upd);
   return g.ou ? launch_update_ou<true, false>(g, t_rel, st, stages, blocks_per_sm, upd)
               : launch_update_ou<false, false>(g, t_rel, st, stages, blocks_per_sm, upd);
+}
+
+bool small_network(const DevNet& g) { return g.nblk <= kSmallBlocks; }
+
+cudaError_t launch_small_steps(const DevNet& g, int32_t n_steps, cudaStream_t st) {
+  static DeviceLaunch cache[kMaxDevices];
+  static std::mutex mu;
+  DeviceLaunch dl;
+  const int most = (int)SmallSmem::bytes(SmallSmem::kN);  // a voxel per neuron
+  const cudaError_t e = device_launch(cache, mu, [&](DeviceLaunch& d) {
+    cudaError_t r = cudaSuccess;
+    for (const void* f : {(const void*)small_steps_kernel<2, false, 512>, (const void*)small_steps_kernel<2, true, 512>,
+                          (const void*)small_steps_kernel<4, false, 512>, (const void*)small_steps_kernel<4, true, 512>,
+                          (const void*)small_steps_kernel<2, false, 1024>, (const void*)small_steps_kernel<2, true, 1024>,
+                          (const void*)small_steps_kernel<4, false, 1024>, (const void*)small_steps_kernel<4, true, 1024>})
+      if (r == cudaSuccess) r = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    d.per_sm = 1;
+    return r;
+  }, &dl);
+  if (e != cudaSuccess) return e;
+  const size_t smem = SmallSmem::bytes(g.nv);
+  const bool few = g.nblk == 1;  // half the threads with twice the registers each, none of them spilled
+  auto run = [&](auto kernel) { kernel<<<1, few ? 512 : 1024, smem, st>>>(g, n_steps); };
+  if (g.nch == 2) {
+    if (g.ou) few ? run(small_steps_kernel<2, true, 512>) : run(small_steps_kernel<2, true, 1024>);
+    else few ? run(small_steps_kernel<2, false, 512>) : run(small_steps_kernel<2, false, 1024>);
+  } else {
+    if (g.ou) few ? run(small_steps_kernel<4, true, 512>) : run(small_steps_kernel<4, true, 1024>);
+    else few ? run(small_steps_kernel<4, false, 512>) : run(small_steps_kernel<4, false, 1024>);
+  }
+  return cudaGetLastError();
 }
 
 cudaError_t prepare_step_kernels() {
