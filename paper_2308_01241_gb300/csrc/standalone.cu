@@ -23,7 +23,7 @@ __global__ void block_count_kernel(const uint32_t* bits, int32_t nblk, int32_t* 
 }  // namespace
 
 // Count + compaction on a DevNet view of caller buffers; scratch holds the
-// block counts [nblk] followed by two 8-byte words (log position, spike sum).
+// block counts [nblk].  There is no spike log and no spike sum here.
 cudaError_t compact_bits(const uint32_t* bits, int64_t n, int32_t* ids, int32_t* count, void* scratch,
                          cudaStream_t st) {
   DevNet g{};
@@ -33,24 +33,19 @@ cudaError_t compact_bits(const uint32_t* bits, int64_t n, int32_t* ids, int32_t*
   g.ntiles = (g.nblk + kCompactBlocksPerTile - 1) / kCompactBlocksPerTile;
   g.flags = const_cast<uint32_t*>(bits);
   g.blk_cnt = (int32_t*)scratch;
-  int64_t* words = (int64_t*)((char*)scratch + compact_scratch_bytes(n) - 16);
-  g.log_pos = words;
-  g.spikes = (unsigned long long*)(words + 1);
   g.log_ids = nullptr;
   g.log_cap = 0;
   g.spk = ids;
   g.n_spk = count;
-  cudaError_t e = cudaMemsetAsync(words, 0, 16, st);
-  if (e != cudaSuccess) return e;
   block_count_kernel<<<(unsigned)((g.nblk * 32 + 255) / 256), 256, 0, st>>>(bits, g.nblk, g.blk_cnt);
-  e = cudaGetLastError();
+  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return launch_spike_compact(g, 0, st);
 }
 
 size_t compact_scratch_bytes(int64_t n) {
   const int64_t nblk = (n + kNeuronsPerBlock - 1) / kNeuronsPerBlock;
-  return (size_t)(((4 * nblk + 15) / 16) * 16 + 16);
+  return (size_t)(((4 * nblk + 15) / 16) * 16);
 }
 
 }  // namespace dtb

@@ -6,7 +6,7 @@
 // real-time loop may forbid calls that can block or synchronise the device,
 // as cudaMalloc and cudaFree can.  A plugin may be handed buffers but have
 // no allocator of its own.  This variant keeps its scratch (the per-block
-// spike counts and two 8-byte words) in a fixed file-scope device array.
+// spike counts) in a fixed file-scope device array.
 // Every GPU that loads the library holds that array until the process
 // exits; no call allocates or frees anything.
 #include <cuda_runtime.h>

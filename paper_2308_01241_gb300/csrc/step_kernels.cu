@@ -827,7 +827,7 @@ __global__ void __launch_bounds__(256) spike_compact_kernel(DevNet g, int32_t t_
   }
 
   if (c) {
-    const int64_t lp = g.log_pos[par];
+    const int64_t lp = g.log_cap ? g.log_pos[par] : 0;
     int pos = base + r0;
 #pragma unroll
     for (int k = 0; k < kWords; k++)
@@ -914,7 +914,7 @@ __global__ void __launch_bounds__(256) spike_compact_kernel(DevNet g, int32_t t_
       *g.call_steps = log_step + 1;
     }
     if (with_items) *g.n_items = ibase + itot;
-    atomicAdd(g.spikes, (unsigned long long)total);
+    if (g.spikes) atomicAdd(g.spikes, (unsigned long long)total);
   }
 }
 
