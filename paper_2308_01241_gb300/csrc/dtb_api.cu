@@ -91,6 +91,7 @@ struct dtb_net {
   uint64_t init_seed = 0;
   double ou_mu = 0;          // initial OU current
   int deliver_blocks = 0;
+  int64_t n_chunks = 0;      // queue mode: chunks of all rows
   int update_stages = 3;     // neuron update pipeline depth
   int update_per_sm = 0;     // neuron update CTAs per SM (0 = as many as fit)
   int schedule = -1;         // requested: -1 by size, 0 compaction after the update, 1 beside the next update
@@ -973,7 +974,7 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
     }
     cb[0] = 0;
     for (int64_t i = 0; i < n; i++) cb[i + 1] = cb[i] + (rp[i + 1] - rp[i] + dtb::kItemEvents - 1) / dtb::kItemEvents;
-    const int64_t n_chunks = cb[n];
+    const int64_t n_chunks = net->n_chunks = cb[n];
     rp.clear();
     rp.shrink_to_fit();
     uint2* pk = (uint2*)net->dalloc(8 * ((size_t)nnz + 1));
@@ -1075,11 +1076,22 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  net->deliver_blocks = sms * dtb::deliver_blocks_per_sm();
+  // CTAs per SM of the deliveries.  Queue mode: as many as have a batch of 8
+  // chunks each when the network fires at 30 Hz, since each CTA without work
+  // costs its launch (us a step with 1 and 8 per SM: 50k neurons 8.4 and 10.2,
+  // 200k with four channels 10.9 and 12.1; 1M at 15 Hz 19.6 with 5, 20.1 with 8;
+  // 2M 33.4 with 4, 32.4 with 8).
+  int per = dtb::deliver_blocks_per_sm();
+  if (g.mode == dtb::kModeQueue) {
+    const double batches = (double)net->n_chunks * 30.0 * 1e-3 * net->dt / 8.0;
+    per = std::max(1, (int)std::min((double)per, std::ceil(batches / sms)));
+  }
+  net->deliver_blocks = sms * per;
   net->sms = sms;
-  // bins mode: two stages, so that three CTAs (with their arrival sums and
-  // staged bins) fit on an SM
-  net->update_stages = g.nch == 2 && g.mode != dtb::kModeBins ? 3 : 2;
+  // Two stages, so that three CTAs fit on an SM in the queue and bins modes
+  // (queue mode, us a step with two and three: 20.1 and 21.0 at 1M neurons, 32.4
+  // and 33.3 at 2M, 58.6 and 61.0 at 3M)
+  net->update_stages = g.nch == 2 && g.mode == dtb::kModeRing ? 3 : 2;
   net->beside = g.nblk <= kBesideMaxBlocks;
   *out = net;
   return DTB_OK;
@@ -1492,7 +1504,7 @@ dtb_status dtb_autotune(dtb_net* net, int32_t n_steps, int32_t* chosen) {
     float ms = 0;
     DTB_CUDA(cudaEventElapsedTime(&ms, e0, e1));
     net->t += n_steps;
-  net->log_par = (int)(net->t & 1);
+    net->log_par = (int)(net->t & 1);
     if (ms < best) {
       best = ms;
       win = c;
