@@ -193,6 +193,7 @@ struct DevNet {
   // their arrival step, qcnt [D][kSubQueues] their counts; the neuron update that
   // consumes a step's arrivals empties its queues).  Bins mode: one queue a step
   int32_t mode;
+  int32_t keep_state;    // state and accumulators fit the L2 cache: no evict-first hint on them
   int32_t n_sub;  // queues per arrival step
   int64_t qcap;   // entries of one
   unsigned long long* q;
@@ -272,6 +273,12 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
 __device__ __forceinline__ uint64_t l2_evict_first() {
   uint64_t p;
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+  return p;
+}
+// The policy of plain loads and stores, for the same instructions.
+__device__ __forceinline__ uint64_t l2_evict_normal() {
+  uint64_t p;
+  asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
   return p;
 }
 __device__ __forceinline__ void bulk_g2s_hint(void* dst, const void* src, uint32_t bytes, uint64_t* bar,

@@ -394,7 +394,9 @@ __global__ void __launch_bounds__(kUpdateThreads, BINS || (NCH == 2 && !OU) ? 3 
   // again for the deliveries of step x + 1 on, which come after this kernel
   if (do_j && g.mode && blockIdx.x == 0 && tid < g.n_sub) g.qcnt[((x % g.D) * g.n_sub + tid) * kQcntStride] = 0;
 
-  const uint64_t once = l2_evict_first();  // state is read and written once per step
+  // state is read and written once per step: it makes room for the accumulators
+  // and queues, unless all of it fits (then it is the synapses that pass through)
+  const uint64_t once = !BINS && g.keep_state ? l2_evict_normal() : l2_evict_first();
   auto issue = [&](int k) {  // one thread: bulk loads of my k-th tile into stage k % S
     uint64_t* b = &bar[k % S];
     const int tl = tile_of(k);
