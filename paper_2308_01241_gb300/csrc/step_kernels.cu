@@ -548,13 +548,9 @@ __global__ void __launch_bounds__(kUpdateThreads, BINS || (NCH == 2 && !OU) ? 3 
     Quad s;
     s.ref4 = reinterpret_cast<const uint32_t*>(st + St::kRef)[tid];
     int4 A4[NCH];
-    uint32_t held = 0;  // channels whose accumulators hold events: only those are cleared below
     if (!BINS) {
 #pragma unroll
-      for (int cc = 0; cc < NCH; cc++) {
-        A4[cc] = reinterpret_cast<const int4*>(st + St::kAcc + cc * 4096)[tid];
-        if (A4[cc].x | A4[cc].y | A4[cc].z | A4[cc].w) held |= 1u << cc;
-      }
+      for (int cc = 0; cc < NCH; cc++) A4[cc] = reinterpret_cast<const int4*>(st + St::kAcc + cc * 4096)[tid];
     }
     const float4 I4 = OU ? reinterpret_cast<const float4*>(st + St::kI)[tid] : make_float4(0.f, 0.f, 0.f, 0.f);
     const uint32_t ni4 = reinterpret_cast<const uint32_t*>(st + St::kNit)[tid];
@@ -620,9 +616,13 @@ __global__ void __launch_bounds__(kUpdateThreads, BINS || (NCH == 2 && !OU) ? 3 
         st_hint(reinterpret_cast<float4*>(g.j + q * np + i0), make_float4(s.J[q][0], s.J[q][1], s.J[q][2], s.J[q][3]),
                 once);
       if (!BINS) {
+        // all of them, also where nothing had arrived: a sector of which one
+        // thread's half is written is read again before it leaves the cache
+        // (clearing only what was not zero: 18.5 us a step for 18.2 at 1M
+        // neurons, 30.4 for 29.8 at 2M, 81.3 for 74.5 at 4M in ring mode)
 #pragma unroll
         for (int cc = 0; cc < NCH; cc++)
-          if ((held >> cc) & 1u) *reinterpret_cast<int4*>(acc_slot + cc * np + i0) = make_int4(0, 0, 0, 0);
+          st_hint(reinterpret_cast<float4*>(acc_slot + cc * np + i0), make_float4(0.f, 0.f, 0.f, 0.f), once);
       }
     }
     // spike bits, and the tile's spikes and work items: the warp that is the
