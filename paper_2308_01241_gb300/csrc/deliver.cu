@@ -28,15 +28,17 @@ __device__ __forceinline__ int32_t stored_weight(const void* w, int64_t e, int s
   return (int32_t)__ldg(reinterpret_cast<const signed char*>(w) + e) * (1 << shift);
 }
 
-// Ring delivery: one warp per work item (up to 512 synapses of one spiking row;
-// grid-stride over the item list), lanes stride over the item, four synapses
-// in flight per lane.  The add is a fire-and-forget reduction at L2, so the
-// order of adds does not matter.
+// Ring delivery: one warp per piece of a spiking row (up to 512 synapses;
+// grid-stride over the list that the neuron update left, so nothing waits for
+// the compaction), lanes stride over the piece, four synapses in flight per lane.
+// The add is a fire-and-forget reduction at L2, so the order of adds does not
+// matter.
 template <int WFMT, int NCH>
 __global__ void __launch_bounds__(256, 8) spike_deliver_kernel(DevNet g, int32_t t_rel) {
   const int64_t t = *g.t_base + t_rel;
   const int32_t tm = (int32_t)(t % g.D);
-  const int32_t n_items = *g.n_items;
+  const int n_list = (int)g.chunk_cnt[t % 3];
+  const ulonglong2* list = g.row_list + (t & 1) * g.list_cap;
   const int lane = threadIdx.x & 31;
   const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -45,10 +47,10 @@ __global__ void __launch_bounds__(256, 8) spike_deliver_kernel(DevNet g, int32_t
   __shared__ unsigned long long s_ev;  // one events atomic per block, not per warp
   if (threadIdx.x == 0) s_ev = 0;
   __syncthreads();
-  for (int64_t ii = gw; ii < n_items; ii += nw) {
-    const WorkItem item = g.items[ii];
-    const int32_t s = item.src;
-    const int64_t r0 = item.e0, r1 = r0 + item.len;
+  for (int64_t ii = gw; ii < n_list; ii += nw) {
+    const ulonglong2 piece = list[ii];
+    const int32_t s = (int32_t)(uint32_t)piece.y;
+    const int64_t r0 = (int64_t)piece.x, r1 = r0 + (int64_t)(piece.y >> 32);
     ev += (unsigned long long)(r1 - r0);
     const int shift = WFMT == 3 ? g.wshift + (g.row_shift ? g.row_shift[s] : 0) : g.wshift;
     for (int64_t e0 = r0 + lane; e0 < r1; e0 += 4 * 32) {

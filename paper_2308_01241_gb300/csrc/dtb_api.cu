@@ -96,7 +96,7 @@ struct dtb_net {
   uint64_t init_seed = 0;
   double ou_mu = 0;          // initial OU current
   int deliver_blocks = 0;
-  int64_t n_chunks = 0;      // queue mode: chunks of all rows
+  int64_t n_chunks = 0;      // queue and ring mode: chunks of all rows, at most
   int update_stages = 3;     // neuron update pipeline depth
   int update_per_sm = 0;     // neuron update CTAs per SM (0 = as many as fit)
   int schedule = -1;         // requested: -1 by size, 0 compaction after the update, 1 beside the next update
@@ -324,9 +324,9 @@ dtb_status ensure_step_off(dtb_net* net, int64_t n_steps) {
 //   s1: update(t), bold(t-2) -> compact(t) -> deliver(t)
 // so compact(t) runs beside update(t + 1).  The two write different copies of
 // the spike bits and block counts (the step's index parity); update(t + 2)
-// reuses compact(t)'s copy only after it.  In the queue mode the update lists the
-// delivery's work itself and nothing waits for the compaction (which then only
-// feeds the spike log and the BOLD step):
+// reuses compact(t)'s copy only after it.  In the queue and ring modes the update
+// lists the delivery's work itself and nothing waits for the compaction (which
+// then only feeds the spike log and the BOLD step):
 //   s1: update(t) -> deliver(t)
 //   s3: update(t) -> compact(t) -> bold(t)   [with net->beside; else compact(t) on s0]
 // update(t) still consumes the arrivals at t - 1 after every delivery that
@@ -372,7 +372,7 @@ dtb_status enqueue_range(dtb_net* net, int32_t k, bool head, cudaEvent_t* tev = 
     const bool first = head && s == 0;
     if (q && s >= 2) DTB_CUDA(cudaStreamWaitEvent(s0, evR[(s - 2) & 1], 0));
     if (bins && s >= 1) DTB_CUDA(cudaStreamWaitEvent(s0, evR[(s - 1) & 1], 0));
-    if (s >= 2 && (beside || q)) DTB_CUDA(cudaStreamWaitEvent(s0, evD[(s - 2) & 1], 0));  // deliver(s-2)
+    if (s >= 2 && (beside || !bins)) DTB_CUDA(cudaStreamWaitEvent(s0, evD[(s - 2) & 1], 0));  // deliver(s-2)
     if (s >= 2 && beside) DTB_CUDA(cudaStreamWaitEvent(s0, evC[(s - 2) & 1], 0));         // compact(s-2)
     if (bins) {
       if (s >= 1) DTB_CUDA(cudaStreamWaitEvent(s2, evF, 0));               // update(s-1)
@@ -388,16 +388,16 @@ dtb_status enqueue_range(dtb_net* net, int32_t k, bool head, cudaEvent_t* tev = 
     DTB_CUDA(mark(s, 0, 1, s0));
     DTB_CUDA(cudaEventRecord(evF, s0));
     // the compaction: after the update on s0, or beside the next update on s1
-    // (there deliver(s-1) precedes it on its own stream) or, in the queue mode, s3
-    cudaStream_t sc = !beside ? s0 : q ? s3 : s1;
+    // (there deliver(s-1) precedes it on its own stream) or, but in bins mode, s3
+    cudaStream_t sc = !beside ? s0 : bins ? s1 : s3;
     if (beside) DTB_CUDA(cudaStreamWaitEvent(sc, evF, 0));
-    if (s >= 1 && !beside && !q) DTB_CUDA(cudaStreamWaitEvent(s0, evD[(s - 1) & 1], 0));
+    if (s >= 1 && !beside && bins) DTB_CUDA(cudaStreamWaitEvent(s0, evD[(s - 1) & 1], 0));
     if (s >= 2) DTB_CUDA(cudaStreamWaitEvent(sc, evB[(s - 2) & 1], 0));
     DTB_CUDA(mark(s, 1, 0, sc));
     DTB_CUDA(dtb::launch_spike_compact(step_view(net, s), s, sc));
     DTB_CUDA(mark(s, 1, 1, sc));
     DTB_CUDA(cudaEventRecord(evC[s & 1], sc));
-    if (q) DTB_CUDA(cudaStreamWaitEvent(s1, evF, 0));
+    if (!bins) DTB_CUDA(cudaStreamWaitEvent(s1, evF, 0));
     else if (!beside) DTB_CUDA(cudaStreamWaitEvent(s1, evC[s & 1], 0));
     DTB_CUDA(mark(s, 2, 0, s1));
     DTB_CUDA(dtb::launch_spike_deliver(step_view(net, s), s, net->deliver_blocks, s1));
@@ -907,21 +907,23 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
   }
 
   // delivery work items: at most one per spike plus one per kItemEvents synapses
-  // (queue mode: chunks, listed by the neuron update)
+  // (queue and ring mode: listed by the neuron update)
   {
     const int64_t cap = n + nnz / dtb::kItemEvents + 1;
     if (cap >= ((int64_t)1 << 31)) {
       delete net;
       return fail(DTB_EINVAL, "too many delivery work items for int32 counts");
     }
-    if (g.mode == dtb::kModeQueue) {
-      g.list_cap = (cap + 63) & ~(int64_t)63;
-      g.chunk_list = (uint32_t*)net->dalloc(4 * 2 * (size_t)g.list_cap);
-      g.chunk_cnt = (uint32_t*)net->dalloc(16);
-    } else {
+    if (g.mode == dtb::kModeBins) {
       g.items = (dtb::WorkItem*)net->dalloc(sizeof(dtb::WorkItem) * (size_t)cap);
+    } else {
+      g.list_cap = (cap + 63) & ~(int64_t)63;
+      if (g.mode == dtb::kModeQueue) g.chunk_list = (uint32_t*)net->dalloc(4 * 2 * (size_t)g.list_cap);
+      else g.row_list = (ulonglong2*)net->dalloc(16 * 2 * (size_t)g.list_cap);
+      g.chunk_cnt = (uint32_t*)net->dalloc(16);
+      net->n_chunks = cap;
     }
-    if (g.mode == dtb::kModeQueue ? !g.chunk_list || !g.chunk_cnt : !g.items) {
+    if (g.mode == dtb::kModeBins ? !g.items : !g.chunk_cnt || (!g.chunk_list && !g.row_list)) {
       delete net;
       return fail(DTB_ENOMEM, "delivery work items");
     }
@@ -1084,22 +1086,27 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  // CTAs per SM of the deliveries.  Queue mode: as many as have a batch of 8
+  // CTAs per SM of the deliveries.  But in bins mode: as many as have a batch of 8
   // chunks each when the network fires at 30 Hz, since each CTA without work
   // costs its launch (us a step with 1 and 8 per SM: 50k neurons 8.4 and 10.2,
   // 200k with four channels 10.9 and 12.1; 1M at 15 Hz 19.6 with 5, 20.1 with 8;
   // 2M 33.4 with 4, 32.4 with 8).
+  // In ring mode two at most: its reductions miss the cache and hold up the
+  // neuron update beside them (us a step with 1, 2, 3 and 8: 2M at 15 Hz 38.5,
+  // 41.2, 42.5, 42.6; 2M at 30 Hz 67.1, 66.1, 66.5, 68.2; 1.3M at 30 Hz 44.6,
+  // 42.3, 41.0, 43.1; 4M at 7 Hz 69.3, 72.8, 74.1, 74.5).
   int per = dtb::deliver_blocks_per_sm();
-  if (g.mode == dtb::kModeQueue) {
+  if (g.mode != dtb::kModeBins) {
     const double batches = (double)net->n_chunks * 30.0 * 1e-3 * net->dt / 8.0;
-    per = std::max(1, (int)std::min((double)per, std::ceil(batches / sms)));
+    const int most = g.mode == dtb::kModeRing ? std::min(per, 2) : per;
+    per = std::max(1, (int)std::min((double)most, std::ceil(batches / sms)));
   }
   net->deliver_blocks = sms * per;
   net->sms = sms;
-  // Two stages, so that three CTAs fit on an SM in the queue and bins modes
-  // (queue mode, us a step with two and three: 20.1 and 21.0 at 1M neurons, 32.4
-  // and 33.3 at 2M, 58.6 and 61.0 at 3M)
-  net->update_stages = g.nch == 2 && g.mode == dtb::kModeRing ? 3 : 2;
+  // Two stages, so that three CTAs fit on an SM (us a step with two and three,
+  // queue mode: 20.1 and 21.0 at 1M neurons, 32.4 and 33.3 at 2M, 58.6 and 61.0 at
+  // 3M; ring mode: 24.5 and 24.1 at 1M, 40.8 and 42.7 at 2M)
+  net->update_stages = 2;
   net->beside = g.nblk <= kBesideMaxBlocks;
   *out = net;
   return DTB_OK;

@@ -64,6 +64,11 @@ struct __align__(16) WorkItem {
   int32_t pad;
 };
 
+// Ring mode: the source and length of a listed piece of a row.
+__device__ __forceinline__ unsigned long long row_piece(int32_t src, int len) {
+  return (unsigned long long)(uint32_t)src | (unsigned long long)len << 32;
+}
+
 // Run tables of the packed synapse records (queue mode, and bins mode with
 // 16-bit weight codes).  Every chunk of kItemEvents synapses of a row is sorted
 // at creation by delay, then target; a run is a stretch of one chunk whose
@@ -155,11 +160,13 @@ struct DevNet {
   const int64_t* chunk_base;  // [n+1] first chunk of each row (with syn_pack)
   const int64_t* run_ptr;     // [chunks+1] first run of each chunk
   // queue mode: the chunks, and the list of those whose neurons fired, in no
-  // order, that the neuron update leaves for the delivery.  Steps alternate
-  // between two lists of list_cap entries; the counts are at t mod 3 (the update
-  // of step t clears the next step's, which the delivery of step t - 2 read)
+  // order, that the neuron update leaves for the delivery; ring mode: a list of
+  // the rows' pieces (first synapse, row_piece).  Steps alternate between two
+  // lists of list_cap entries; the counts are at t mod 3 (the update of step t
+  // clears the next step's, which the delivery of step t - 2 read)
   const ChunkInfo* chunks;
   uint32_t* chunk_list;
+  ulonglong2* row_list;
   uint32_t* chunk_cnt;
   int64_t list_cap;
   const uint32_t* runs;       // run records
@@ -169,8 +176,8 @@ struct DevNet {
   int32_t* spk;     // [2][spk_par] by step parity, as n_spk and log_pos
   int32_t* n_spk;
   int64_t spk_par;
-  // delivery work items of the current step, ascending by source; blk_items
-  // [nblk] per-block counts, n_items their total
+  // bins mode: delivery work items of the current step, ascending by source;
+  // blk_items [nblk] per-block counts, n_items their total
   int32_t* blk_items;
   WorkItem* items;
   const uint8_t* nitem;  // [npad] work items of each neuron's row (0 beyond n); used when nitem_ok

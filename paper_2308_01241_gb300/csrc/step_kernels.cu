@@ -302,8 +302,8 @@ struct Stage {
   // registers, so that three CTAs fit on an SM
   static constexpr uint32_t kV = 0, kJ = 4096, kRef = BINS ? 4096 : kJ + 4 * 4096, kAcc = kRef + 1024;
   static constexpr uint32_t kI = kAcc + (BINS ? 0 : NCH * 4096);
-  static constexpr uint32_t kNit = kI + (OU ? 4096 : 0);  // work items per neuron (1 B each)
-  static constexpr uint32_t kBytes = kNit + kNeuronsPerBlock;  // one tile
+  static constexpr uint32_t kNit = kI + (OU ? 4096 : 0);  // bins mode: work items per neuron (1 B each)
+  static constexpr uint32_t kBytes = kNit + (BINS ? kNeuronsPerBlock : 0);  // one tile
   // bins mode: the region's arrival sums and its staged bin sit in front of the stages
   static constexpr uint32_t kRegionAcc = BINS ? NCH * kRegionNeurons * 4 : 0;
   static constexpr uint32_t kFront = BINS ? kRegionAcc + kEvBufWords * 4 : 0;
@@ -316,15 +316,18 @@ __device__ __forceinline__ uint32_t taken_add(uint32_t* p) {
   return old;
 }
 
-// Queue mode: a warp's spiking neurons (id, or -1 for a lane without one) as
-// chunks on the delivery's list.
-__device__ __forceinline__ void list_chunks(const DevNet& g, int32_t id, uint32_t* list, uint32_t* cnt, int lane) {
-  int64_t cb = 0;
-  int nc = 0;
+// A warp's spiking neurons (id, or -1 for a lane without one) on the delivery's
+// list of step t: queue mode, the chunks of their rows; ring mode, their rows in
+// pieces of kItemEvents synapses.
+__device__ __forceinline__ void list_work(const DevNet& g, int32_t id, int64_t t, int lane) {
+  const bool rows = g.row_list != nullptr;
+  int64_t cb = 0, len = 0;
   if (id >= 0) {
-    cb = __ldg(g.chunk_base + id);
-    nc = (int)(__ldg(g.chunk_base + id + 1) - cb);
+    const int64_t* p = (rows ? g.row_ptr : g.chunk_base) + id;
+    cb = __ldg(p);
+    len = __ldg(p + 1) - cb;
   }
+  const int nc = (int)(rows ? (len + kItemEvents - 1) / kItemEvents : len);
   int end = nc;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -332,9 +335,16 @@ __device__ __forceinline__ void list_chunks(const DevNet& g, int32_t id, uint32_
     if (lane >= o) end += y;
   }
   uint32_t base = 0;
-  if (lane == 31 && end > 0) base = atomicAdd(cnt, (uint32_t)end);
+  if (lane == 31 && end > 0) base = atomicAdd(g.chunk_cnt + t % 3, (uint32_t)end);
   base = __shfl_sync(0xFFFFFFFFu, base, 31) + (uint32_t)(end - nc);
-  for (int k = 0; k < nc; k++) list[base + k] = (uint32_t)(cb + k);
+  const int64_t at = (t & 1) * g.list_cap + base;
+  if (rows) {
+    for (int k = 0; k < nc; k++)
+      g.row_list[at + k] = make_ulonglong2((unsigned long long)(cb + (int64_t)k * kItemEvents),
+                                           row_piece(id, (int)min(len - (int64_t)k * kItemEvents, (int64_t)kItemEvents)));
+  } else {
+    for (int k = 0; k < nc; k++) g.chunk_list[at + k] = (uint32_t)(cb + k);
+  }
 }
 constexpr int kSpikeList = 1024;  // spikes of a CTA held in shared memory until its end
 
@@ -363,7 +373,7 @@ __global__ void __launch_bounds__(kUpdateThreads, BINS || (NCH == 2 && !OU) ? 3 
   // the tiles' constants, in a ring of their own: it is deep enough that a
   // refill never meets a warp still reading, so no thread holds them in registers
   __shared__ __align__(16) VoxConst s_vc[kSlots];
-  __shared__ int32_t s_spk[BINS ? 1 : kSpikeList];  // queue mode: the CTA's spikes
+  __shared__ int32_t s_spk[BINS ? 1 : kSpikeList];  // ring and queue modes: the CTA's spikes
   __shared__ int s_nspk;
   __shared__ uint32_t s_done[kSlots];   // warps done with the tile << 28 | its spikes
   __shared__ uint32_t s_items[kSlots];  // its delivery work items
@@ -415,7 +425,7 @@ __global__ void __launch_bounds__(kUpdateThreads, BINS || (NCH == 2 && !OU) ? 3 
     }
     if (OU) bulk_g2s_hint(st + St::kI, g.Iou + base, 4096, b, once);
     bulk_g2s(&s_vc[k % kSlots], g.tile_vc + tl, sizeof(VoxConst), b);
-    bulk_g2s_hint(st + St::kNit, g.nitem + base, kNeuronsPerBlock, b, once);
+    if (BINS) bulk_g2s_hint(st + St::kNit, g.nitem + base, kNeuronsPerBlock, b, once);
   };
   // bins mode: the bin of my m-th region, parity of step x
   const int par = (int)(x & 1);
@@ -443,9 +453,7 @@ __global__ void __launch_bounds__(kUpdateThreads, BINS || (NCH == 2 && !OU) ? 3 
     s_done[tid] = 0;
     s_items[tid] = 0;
   }
-  const bool listing = !BINS && do_v && g.mode == kModeQueue;
-  uint32_t* list = listing ? g.chunk_list + (t & 1) * g.list_cap : nullptr;
-  uint32_t* list_cnt = listing ? g.chunk_cnt + t % 3 : nullptr;
+  const bool listing = !BINS && do_v;
   if (tid == 0) {
     s_nspk = 0;
     if (listing && blockIdx.x == 0) g.chunk_cnt[(t + 1) % 3] = 0;
@@ -553,7 +561,7 @@ __global__ void __launch_bounds__(kUpdateThreads, BINS || (NCH == 2 && !OU) ? 3 
       for (int cc = 0; cc < NCH; cc++) A4[cc] = reinterpret_cast<const int4*>(st + St::kAcc + cc * 4096)[tid];
     }
     const float4 I4 = OU ? reinterpret_cast<const float4*>(st + St::kI)[tid] : make_float4(0.f, 0.f, 0.f, 0.f);
-    const uint32_t ni4 = reinterpret_cast<const uint32_t*>(st + St::kNit)[tid];
+    const uint32_t ni4 = BINS ? reinterpret_cast<const uint32_t*>(st + St::kNit)[tid] : 0u;
     const VoxConst* vc = &s_vc[k % kSlots];
     const bool first_vox = tid * 4 + 3 < vc->n_first;
     __syncwarp();
@@ -656,22 +664,24 @@ __global__ void __launch_bounds__(kUpdateThreads, BINS || (NCH == 2 && !OU) ? 3 
         } else {  // no room left (rare): listed here, and the slots marked empty
           for (int k = at + lane; k < min(at + all, kSpikeList); k += 32) s_spk[k] = -1;
 #pragma unroll 1
-          for (int q = 0; q < 4; q++) list_chunks(g, (nib >> q) & 1u ? (int32_t)i0 + q : -1, list, list_cnt, lane);
+          for (int q = 0; q < 4; q++) list_work(g, (nib >> q) & 1u ? (int32_t)i0 + q : -1, t, lane);
         }
       }
-#pragma unroll
-      for (int q = 0; q < 4; q++)
-        if (!listing && ((nib >> q) & 1u)) {
-          if (g.nitem_ok) {
-            nit += (int)((ni4 >> (8 * q)) & 0xFFu);
-          } else {
-            const int64_t len = g.row_ptr[i0 + q + 1] - g.row_ptr[i0 + q];
-            nit += (int)((len + kItemEvents - 1) / kItemEvents);
-          }
-        }
       cnt = __reduce_add_sync(0xFFFFFFFFu, __popc(nib));
-      nit = __reduce_add_sync(0xFFFFFFFFu, nit);
-      if (lane == 0) atomicAdd(&s_items[k % kSlots], (uint32_t)nit);
+      if (BINS) {
+#pragma unroll
+        for (int q = 0; q < 4; q++)
+          if ((nib >> q) & 1u) {
+            if (g.nitem_ok) {
+              nit += (int)((ni4 >> (8 * q)) & 0xFFu);
+            } else {
+              const int64_t len = g.row_ptr[i0 + q + 1] - g.row_ptr[i0 + q];
+              nit += (int)((len + kItemEvents - 1) / kItemEvents);
+            }
+          }
+        nit = __reduce_add_sync(0xFFFFFFFFu, nit);
+        if (lane == 0) atomicAdd(&s_items[k % kSlots], (uint32_t)nit);
+      }
     }
     if ((lane & 7) == 0) g.flags[i0 >> 5] = word;  // i0 of lane 8q is the first neuron of word q
     if (lane == 0) {
@@ -680,8 +690,10 @@ __global__ void __launch_bounds__(kUpdateThreads, BINS || (NCH == 2 && !OU) ? 3 
       if (old >> 28 == kWarps - 1) {
         __threadfence_block();
         g.blk_cnt[tile] = (int32_t)(old & 0xFFFFu) + cnt;
-        g.blk_items[tile] = (int32_t)s_items[k % kSlots];
-        s_items[k % kSlots] = 0;
+        if (BINS) {
+          g.blk_items[tile] = (int32_t)s_items[k % kSlots];
+          s_items[k % kSlots] = 0;
+        }
         s_done[k % kSlots] = 0;
       }
     }
@@ -690,7 +702,7 @@ __global__ void __launch_bounds__(kUpdateThreads, BINS || (NCH == 2 && !OU) ? 3 
   const bool gave_up = __syncthreads_or(bad);
   if (listing) {
     const int n_spk = min(s_nspk, kSpikeList);
-    for (int k = tid & ~31; k < n_spk; k += kThr) list_chunks(g, k + lane < n_spk ? s_spk[k + lane] : -1, list, list_cnt, lane);
+    for (int k = tid & ~31; k < n_spk; k += kThr) list_work(g, k + lane < n_spk ? s_spk[k + lane] : -1, t, lane);
   }
   if (gave_up && tid == 0) {
     for (int q = 0; q < S; q++) {
@@ -1210,6 +1222,7 @@ __global__ void __launch_bounds__(MAXT, 1) small_steps_kernel(DevNet g, int32_t 
     g.vox_spikes[my_vox] += vox_total;
   }
   if (lane == 0 && events) atomicAdd(g.events, events);
+  if (tid < 3) g.chunk_cnt[tid] = 0;  // the lists of a network that is stepped by the other kernels next
   if (tid == nthr) {
     g.log_pos[0] = g.log_pos[1] = log_pos;
     if (trunc) *g.log_trunc = 1;
