@@ -100,7 +100,8 @@ enum {
 
 /* How delivered events wait out their delay (the results are the same bit for bit;
  * DTB_DELIVER_BINS without a bin_capacity of the caller's keeps the queue layout
- * for networks whose accumulators are at most 24 MiB, and both keep the ring, without
+ * for networks whose accumulators are at most 28 MiB (48 MiB with 32-bit weights, or
+ * with four channels and the OU drive), and both keep the ring, without
  * capacities of the caller's, for networks of at most 3,072 neurons with at most 200
  * synapses per neuron: they are the faster ones there). */
 enum {

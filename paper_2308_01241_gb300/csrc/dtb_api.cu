@@ -70,10 +70,13 @@ constexpr int64_t kKeepBytes = (int64_t)88 << 20;
 // large use the queue layout where bins are asked for (without a bin capacity
 // of the caller's): it stays in the L2 cache beside the neuron state, and one
 // reduction there per event is less work than sorting the events into bins.
-// Step, bins -> queue: 33.1 -> 20.1 us (1M neurons, 15 Hz), 36.4 -> 31.6 (2M);
-// at 5M and 7 Hz the bins are ahead (61.2 against 65.7 us), their accumulator
-// no longer fits.
-constexpr int64_t kQueueMaxBytes = 24 << 20;
+// us a step, bins and queue: 36.4 and 29.8 (2M neurons, 15 Hz), 49.3 and 47.2
+// (3.6M, 7 Hz), 87.4 and 79.5 (3.6M int8, 30 Hz); 51.7 and 56.7 (3.9M, 7 Hz), 61.3
+// and 68.5 (5M, 7 Hz): the accumulators no longer fit.  The bins' kernels are
+// slower with 32-bit weights (8-byte events) and for four channels with the OU
+// drive, where the line lies further out: 87.3 and 68.5 (5M int32, 7 Hz), 195 and
+// 104 (30 Hz), 91.3 and 80.4 (6M int32), 115 and 94 (3M, four channels, OU, 30 Hz).
+constexpr int64_t kQueueMaxBytes = 28 << 20, kQueueMaxBytesWide = 48 << 20;
 constexpr int kBoldLogCap = 1024;
 
 }  // namespace
@@ -746,10 +749,20 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
     g.mode = dtb::kModeRing;
     net->routed = true;
   }
-  if (g.mode == dtb::kModeBins && n <= (int64_t)dtb::kMaxRegions * dtb::kRegionNeurons && d->bin_capacity == 0 &&
-      4 * npad * g.nch <= kQueueMaxBytes) {
-    g.mode = dtb::kModeQueue;
-    net->routed = true;
+  if (g.mode == dtb::kModeBins && n <= (int64_t)dtb::kMaxRegions * dtb::kRegionNeurons && d->bin_capacity == 0) {
+    const bool wide = d->weight_format == DTB_W_INT32 || (g.nch == 4 && d->ou_enable);
+    bool room = 4 * npad * g.nch <= (wide ? kQueueMaxBytesWide : kQueueMaxBytes);
+    if (room && d->weight_format == DTB_W_INT32) {
+      // the queues read packed records, 8 bytes per synapse, which the bins of
+      // 32-bit weights do without: only with room to spare
+      size_t free_b = 0, total_b = 0;
+      room = cudaMemGetInfo(&free_b, &total_b) == cudaSuccess &&
+             (int64_t)free_b >= 24 * std::max<int64_t>(nnz, 0) + ((int64_t)1 << 30);
+    }
+    if (room) {
+      g.mode = dtb::kModeQueue;
+      net->routed = true;
+    }
   }
   net->small = g.mode == dtb::kModeRing && few;
   // V, j, ref and I, and the two accumulators of the queue mode
