@@ -716,13 +716,6 @@ cudaError_t launch_deliver_runs(const DevNet& g, int32_t t_rel, int blocks, cuda
 
 }  // namespace
 
-cudaError_t prepare_bins_kernels() {
-  return share_sm_division(spike_deliver_bins32_kernel<2>, spike_deliver_bins32_kernel<4>, spike_deliver_runs_kernel<0, 2>,
-                           spike_deliver_runs_kernel<2, 2>, spike_deliver_runs_kernel<3, 2>,
-                           spike_deliver_runs_kernel<0, 4>, spike_deliver_runs_kernel<2, 4>,
-                           spike_deliver_runs_kernel<3, 4>, bin_kernel<false>, bin_kernel<true>);
-}
-
 cudaError_t launch_bins_deliver(const DevNet& g, int32_t t_rel, int blocks, cudaStream_t st) {
   if (g.wfmt == 1) {
     return g.nch == 2 ? launch_deliver_32<2>(g, t_rel, blocks, st) : launch_deliver_32<4>(g, t_rel, blocks, st);

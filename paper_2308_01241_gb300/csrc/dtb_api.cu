@@ -1084,7 +1084,6 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
   {
     cudaError_t e2 = dtb::prepare_step_kernels();
     if (e2 == cudaSuccess) e2 = dtb::prepare_deliver_kernels();
-    if (e2 == cudaSuccess) e2 = dtb::prepare_bins_kernels();
     if (e2 != cudaSuccess) {
       delete net;
       return cuda_fail(e2, "kernel attributes");
@@ -1121,6 +1120,7 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
   // 3M; ring mode: 24.5 and 24.1 at 1M, 40.8 and 42.7 at 2M)
   net->update_stages = 2;
   net->beside = g.nblk <= kBesideMaxBlocks;
+  g.beside = net->beside;
   *out = net;
   return DTB_OK;
 }
@@ -1571,6 +1571,7 @@ dtb_status dtb_set_schedule(dtb_net* net, int32_t mode) {
   if (mode < -1 || mode > 1) return fail(DTB_EINVAL, "schedule must be -1, 0 or 1");
   net->schedule = mode;
   net->beside = mode < 0 ? net->g.nblk <= kBesideMaxBlocks : mode == 1;
+  net->g.beside = net->beside;
   net->drop_graphs();  // the schedule is baked into the graphs
   return DTB_OK;
 }

@@ -200,6 +200,7 @@ struct DevNet {
   // their arrival step, qcnt [D][kSubQueues] their counts; the neuron update that
   // consumes a step's arrivals empties its queues).  Bins mode: one queue a step
   int32_t mode;
+  int32_t beside;        // the compaction of a step runs beside the update of the next
   int32_t keep_state;    // state and accumulators fit the L2 cache: no evict-first hint on them
   int32_t n_sub;  // queues per arrival step
   int64_t qcap;   // entries of one

@@ -32,7 +32,6 @@ int deliver_blocks_per_sm();
 // Attributes of the step's kernels on the current device (once per network).
 cudaError_t prepare_step_kernels();
 cudaError_t prepare_deliver_kernels();
-cudaError_t prepare_bins_kernels();
 
 // setup
 cudaError_t launch_init_voltage(const DevNet& g, uint64_t init_seed, cudaStream_t st);
