@@ -1341,6 +1341,19 @@ dtb_status dtb_set_state(dtb_net* net, const float* V, const float* j, const uin
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(e, "dense ring to spill ring");
   }
+  if (!ring && g.mode && t != net->t) {
+    // a ring left unchanged keeps its slots: what had spilled into one (its mark
+    // names an arrival step still to come) now arrives at that slot's next step
+    std::vector<int32_t> old((size_t)g.D), mark((size_t)g.D, 0);
+    DTB_CUDA(cudaMemcpyAsync(old.data(), g.spill_dirty, 4 * (size_t)g.D, cudaMemcpyDeviceToHost, st));
+    DTB_CUDA(cudaStreamSynchronize(st));
+    for (int64_t x = t; x < t + g.D; x++) {
+      const int64_t s = x % g.D, was = net->t + (s - net->t % g.D + g.D) % g.D;
+      if (old[(size_t)s] == dtb::spill_mark(was)) mark[(size_t)s] = dtb::spill_mark(x);
+    }
+    DTB_CUDA(cudaMemcpyAsync(g.spill_dirty, mark.data(), 4 * (size_t)g.D, cudaMemcpyHostToDevice, st));
+    DTB_CUDA(cudaStreamSynchronize(st));  // mark leaves scope
+  }
   if (g.chunk_cnt) DTB_CUDA(cudaMemsetAsync(g.chunk_cnt, 0, 16, st));
   DTB_CUDA(cudaMemcpyAsync(g.t_base, &t, 8, cudaMemcpyHostToDevice, st));
   DTB_CUDA(cudaStreamSynchronize(st));
