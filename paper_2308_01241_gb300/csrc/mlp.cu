@@ -912,7 +912,12 @@ dtb_status dtb_mlp_forward(dtb_mlp* n, const float* d_x, float* d_y, int64_t B, 
   cudaStream_t st = (cudaStream_t)stream;
   cudaError_t e;
   if (n->fused) {
-    e = fused_predict(n, d_x, d_y, B, st);
+    // an output over its own input goes through a buffer: rows that a CTA has
+    // still to read may lie where another one writes
+    const bool over = (uintptr_t)d_y < (uintptr_t)(d_x + B * n->n_in) && (uintptr_t)d_x < (uintptr_t)(d_y + B * n->n_out);
+    e = fused_predict(n, d_x, over ? n->y : d_y, B, st);
+    if (e == cudaSuccess && over)
+      e = cudaMemcpyAsync(d_y, n->y, 4 * (size_t)B * n->n_out, cudaMemcpyDeviceToDevice, st);
   } else {
     e = stage_input(n, d_x, B, st);
     if (e == cudaSuccess) e = forward(n, B, st);
