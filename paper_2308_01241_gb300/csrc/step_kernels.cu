@@ -1312,7 +1312,9 @@ cudaError_t launch_neuron_update(const DevNet& g, int32_t t_rel, cudaStream_t st
               : launch_update_ou<false, false>(g, t_rel, st, stages, blocks_per_sm, upd);
 }
 
-bool small_network(const DevNet& g) { return g.nblk <= kSmallBlocks; }
+// Voxels may be empty, so there can be more of them than neurons: the voxel
+// counts have room in shared memory for one voxel per neuron.
+bool small_network(const DevNet& g) { return g.nblk <= kSmallBlocks && g.nv <= SmallSmem::kN; }
 
 cudaError_t launch_small_steps(const DevNet& g, int32_t n_steps, cudaStream_t st) {
   static DeviceLaunch cache[kMaxDevices];
