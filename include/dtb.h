@@ -103,7 +103,8 @@ enum {
  * for networks whose accumulators are at most 28 MiB (48 MiB with 32-bit weights, or
  * with four channels and the OU drive), and both keep the ring, without
  * capacities of the caller's, for networks of at most 3,072 neurons and 3,072
- * voxels with at most 200 synapses per neuron: they are the faster ones there). */
+ * voxels with at most 200 synapses per neuron and 8,192 in rows of more than 512:
+ * they are the faster ones there). */
 enum {
   DTB_DELIVER_RING = 0,  /* dense ring acc[D][n_channels][N]: every synapse event is one int32
                             reduction into slot (t + d) mod D */

@@ -53,6 +53,13 @@ constexpr int64_t kSmallSteps = 4096;  // steps per launch of a small network (s
 // At 150 the two meet near 100 Hz; 1,000 neurons: 6.8 and 3.3 at 10 Hz, 9.5 and
 // 7.9 at 117 Hz.
 constexpr int64_t kSmallInDegree = 200;
+// Synapses of such a network in rows of more than a delivery work item: a long row
+// holds up its warp, and with it every step in which its neuron fires.  3,000
+// neurons, 60 to 200 synapses each on average, us a step of the launches and of
+// the one CTA: 7.4 and 5.3 with one row of 3,000 (106 Hz), 7.4 and 7.4 with one of
+// 30,000 (103 Hz), 7.0 and 27 with ten of 30,000, 7.1 and 22 with a hundred of
+// 3,000 (74 Hz).
+constexpr int64_t kSmallLongRows = 8192;
 constexpr int kTimedKernels = 5;  // update, compaction, delivery, drain or binning, BOLD
 // Networks of at most this many 1,024-neuron blocks run the compaction of a
 // step beside the neuron update of the next by default: their kernels leave
@@ -744,7 +751,23 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
   // networks (whose steps run in one CTA), the queues where the accumulator fits
   // the cache
   const bool free_layout = d->bin_capacity == 0 && d->event_queue_capacity == 0;
-  const bool few = dtb::small_network(g) && nnz <= kSmallInDegree * n;
+  bool few = dtb::small_network(g) && nnz <= kSmallInDegree * n;
+  if (few) {
+    std::vector<int64_t> rp;
+    const int64_t* r = d->row_ptr;
+    if (d->csr_on_device) {
+      rp.resize((size_t)n + 1);
+      const cudaError_t e = cudaMemcpy(rp.data(), r, 8 * ((size_t)n + 1), cudaMemcpyDeviceToHost);
+      if (e != cudaSuccess) {
+        delete net;
+        return cuda_fail(e, "reading row_ptr");
+      }
+      r = rp.data();
+    }
+    int64_t in_long = 0;
+    for (int64_t i = 0; i < n; i++) in_long += r[i + 1] - r[i] > dtb::kItemEvents ? r[i + 1] - r[i] : 0;
+    few = in_long <= kSmallLongRows;
+  }
   if (g.mode && free_layout && few) {
     g.mode = dtb::kModeRing;
     net->routed = true;
