@@ -1024,20 +1024,19 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
     rp.clear();
     rp.shrink_to_fit();
     uint2* pk = (uint2*)net->dalloc(8 * ((size_t)nnz + 1));
-    uint8_t* dl = (uint8_t*)net->dalloc((size_t)std::max<int64_t>(nnz, 1));
     int64_t* d_cb = (int64_t*)net->dalloc(8 * ((size_t)n + 1));
     int64_t* d_rp = (int64_t*)net->dalloc(8 * ((size_t)n_chunks + 1));
     int32_t* d_cnt = (int32_t*)net->dalloc(4 * (size_t)std::max<int64_t>(n_chunks, 1));
     dtb::ChunkInfo* d_ci = nullptr;
     if (g.mode == dtb::kModeQueue)
       d_ci = (dtb::ChunkInfo*)net->dalloc(sizeof(dtb::ChunkInfo) * (size_t)std::max<int64_t>(n_chunks, 1));
-    if (!pk || !dl || !d_cb || !d_rp || !d_cnt || (g.mode == dtb::kModeQueue && !d_ci)) {
+    if (!pk || !d_cb || !d_rp || !d_cnt || (g.mode == dtb::kModeQueue && !d_ci)) {
       delete net;
       return fail(DTB_ENOMEM, "packed synapse records and run tables");
     }
     g.chunk_base = d_cb;
     e2 = cudaMemcpyAsync(d_cb, cb.data(), 8 * ((size_t)n + 1), cudaMemcpyHostToDevice, st);
-    if (e2 == cudaSuccess) e2 = dtb::launch_pack_fill(g, pk, dl, d_cnt, st);
+    if (e2 == cudaSuccess) e2 = dtb::launch_pack_fill(g, pk, d_cnt, st);
     std::vector<int32_t> cnt((size_t)n_chunks);
     if (e2 == cudaSuccess) e2 = cudaMemcpyAsync(cnt.data(), d_cnt, 4 * (size_t)n_chunks, cudaMemcpyDeviceToHost, st);
     if (e2 == cudaSuccess) e2 = cudaStreamSynchronize(st);
@@ -1057,13 +1056,12 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
       return fail(DTB_ENOMEM, "run tables");
     }
     e2 = cudaMemcpyAsync(d_rp, run_ptr.data(), 8 * ((size_t)n_chunks + 1), cudaMemcpyHostToDevice, st);
-    if (e2 == cudaSuccess) e2 = dtb::launch_run_fill(g, pk, dl, d_rp, d_runs, d_ci, st);
+    if (e2 == cudaSuccess) e2 = dtb::launch_run_fill(g, pk, d_rp, d_runs, d_ci, st);
     if (e2 == cudaSuccess) e2 = cudaStreamSynchronize(st);
     if (e2 != cudaSuccess) {
       delete net;
       return cuda_fail(e2, "run tables");
     }
-    net->dfree(dl);
     g.syn_pack = pk;
     g.run_ptr = d_rp;
     g.runs = d_runs;

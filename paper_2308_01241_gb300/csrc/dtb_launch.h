@@ -64,15 +64,15 @@ int32_t set_last_error(int32_t code, const std::string& msg);
 // Fills the per-synapse delay bytes out [nnz] (after the synapse check).
 cudaError_t launch_delay_fill(const DevNet& g, uint8_t* out, cudaStream_t st);
 // Fills the packed synapse records out [nnz + 1] (queue mode, and bins mode
-// with 16-bit weight codes), after
-// the synapse check, each chunk of a row sorted by delay and target; delays
-// [nnz] receives the records' delays, counts [chunks] each chunk's number of
-// runs (g.chunk_base set).
-cudaError_t launch_pack_fill(const DevNet& g, uint2* out, uint8_t* delays, int32_t* counts, cudaStream_t st);
-// The chunks' run records from the run pointers (and, in bins mode, each
-// packed record's run index; info, when given: the chunks' info).
-cudaError_t launch_run_fill(const DevNet& g, uint2* pack, const uint8_t* delays, const int64_t* run_ptr,
-                            uint32_t* runs, ChunkInfo* info, cudaStream_t st);
+// with 16-bit weight codes), after the synapse check, each chunk of a row
+// sorted by delay and target; counts [chunks] receives each chunk's number of
+// runs (g.chunk_base set).  launch_run_fill completes them.
+cudaError_t launch_pack_fill(const DevNet& g, uint2* out, int32_t* counts, cudaStream_t st);
+// The chunks' run records from the run pointers, and each packed record's run
+// index (bins mode) or accumulator value (queue mode; info, when given: the
+// chunks' info).
+cudaError_t launch_run_fill(const DevNet& g, uint2* pack, const int64_t* run_ptr, uint32_t* runs, ChunkInfo* info,
+                            cudaStream_t st);
 cudaError_t launch_bounded_wait(long long max_cycles, int32_t arrive, int32_t* status, cudaStream_t st);
 cudaError_t launch_item_count(const DevNet& g, uint8_t* out, int32_t* too_long, cudaStream_t st);
 cudaError_t launch_philox(const uint32_t* ctr, const uint32_t* key, uint32_t* out, int64_t n, cudaStream_t st);

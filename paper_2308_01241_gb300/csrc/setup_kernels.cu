@@ -170,13 +170,16 @@ struct RunHeads {
 
 // Warp per row: every synapse as a packed record, each chunk of kItemEvents
 // synapses (one delivery work item) sorted by delay (from the voxel-pair
-// table) and target, so that its events wait in few places (runs).  delays
-// receives the sorted records' delays and counts[chunk_base[row] + k] the
-// chunk's runs.  A sort key is delay | target | class | weight code, or for
-// 32-bit weights the place in the chunk, from which the weight is read again.
+// table) and target, so that its events wait in few places (runs).
+// counts[chunk_base[row] + k] receives the chunk's runs.  A record is (word,
+// weight code | delay << 16) until run_fill replaces the second word; 32-bit
+// weights leave no room for the delay, which run_fill then looks up again (a
+// buffer of the delays was another byte per synapse on top of all the rest).
+// A sort key is delay | target | class | weight code, or for 32-bit weights the
+// place in the chunk, from which the weight is read again.
 // The order of a row's synapses changes no result: the sums are exact integers.
 template <int WFMT>
-__global__ void __launch_bounds__(256) pack_fill_kernel(DevNet g, uint2* out, uint8_t* delays, int32_t* counts) {
+__global__ void __launch_bounds__(256) pack_fill_kernel(DevNet g, uint2* out, int32_t* counts) {
   constexpr int R = kItemEvents / 32;
   const int lane = threadIdx.x & 31;
   const bool bins = g.mode == kModeBins;
@@ -215,9 +218,8 @@ __global__ void __launch_bounds__(256) pack_fill_kernel(DevNet g, uint2* out, ui
         runs += __popc(rh.round(k, valid, r * 32 + lane, lane, !bins));
         if (valid) {
           const uint32_t low = (uint32_t)(v[r] & 0xFFFFu);
-          const uint32_t code = WFMT == 1 ? weight_code<1>(g.w, c0 + low, 0) : low;
-          out[e] = make_uint2(word, bins ? code : (uint32_t)decode_weight(code, WFMT, g.wshift));
-          delays[e] = (uint8_t)d;
+          out[e] = make_uint2(word, WFMT == 1 ? (uint32_t)decode_weight(weight_code<1>(g.w, c0 + low, 0), 1, g.wshift)
+                                              : low | (d << 16));
         }
       }
       if (lane == 0) counts[chunk] = runs;
@@ -226,16 +228,17 @@ __global__ void __launch_bounds__(256) pack_fill_kernel(DevNet g, uint2* out, ui
 }
 
 // Warp per row, after pack_fill and the run pointers: every chunk's run
-// records (key | start << 14 | (length - 1) << 23) at runs[run_ptr[chunk]..],
-// in bins mode each packed record's run index above its weight code, and in
-// the queue mode the chunk's info.
-__global__ void __launch_bounds__(256) run_fill_kernel(DevNet g, uint2* pack, const uint8_t* delays,
-                                                       const int64_t* run_ptr, uint32_t* runs, ChunkInfo* info) {
+// records (key | start << 14 | (length - 1) << 23) at runs[run_ptr[chunk]..];
+// in bins mode each packed record's run index above its weight code, in the
+// queue mode its accumulator value, and the chunk's info.
+__global__ void __launch_bounds__(256) run_fill_kernel(DevNet g, uint2* pack, const int64_t* run_ptr, uint32_t* runs,
+                                                       ChunkInfo* info) {
   const int lane = threadIdx.x & 31;
-  const bool bins = g.mode == kModeBins;
+  const bool bins = g.mode == kModeBins, wide = g.wfmt == 1;
   const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t s = gw; s < g.n; s += nw) {
+    const uint8_t* drow = g.delay + (int64_t)voxel_of(g, (int32_t)s) * g.nv;
     const int64_t r0 = g.row_ptr[s], r1 = g.row_ptr[s + 1];
     int64_t chunk = g.chunk_base[s];
     for (int64_t c0 = r0; c0 < r1; c0 += kItemEvents, chunk++) {
@@ -248,11 +251,14 @@ __global__ void __launch_bounds__(256) run_fill_kernel(DevNet g, uint2* pack, co
         const int64_t e = c0 + p + lane;
         const bool valid = p + lane < n;
         const uint2 rec = valid ? pack[e] : make_uint2(0u, 0u);
-        const uint32_t k = valid ? synapse_run_key(rec.x, delays[e], bins) : 0xFFFFFFFFu;
+        const uint32_t d = !wide ? (rec.y >> 16) & 0xFFu : valid ? drow[voxel_of(g, (int32_t)(rec.x & 0x3FFFFFFFu))] : 0u;
+        const uint32_t k = valid ? synapse_run_key(rec.x, d, bins) : 0xFFFFFFFFu;
         const unsigned heads = rh.round(k, valid, p + lane, lane, !bins);
         const int idx = before + __popc(heads & (0xFFFFFFFFu >> (31 - lane))) - 1;
         if ((heads >> lane) & 1u) out[idx] = k | ((uint32_t)(p + lane) << 14);
-        if (bins && valid) pack[e].y = (rec.y & 0xFFFFu) | ((uint32_t)idx << 16);
+        if (valid && !wide)
+          pack[e].y = bins ? (rec.y & 0xFFFFu) | ((uint32_t)idx << 16)
+                           : (uint32_t)decode_weight(rec.y & 0xFFFFu, g.wfmt, g.wshift);
         before += __popc(heads);
         n1 += __popc(__ballot_sync(0xFFFFFFFFu, valid && (k & kRunRegion)));
       }
@@ -573,25 +579,25 @@ cudaError_t launch_delay_fill(const DevNet& g, uint8_t* out, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_pack_fill(const DevNet& g, uint2* out, uint8_t* delays, int32_t* counts, cudaStream_t st) {
+cudaError_t launch_pack_fill(const DevNet& g, uint2* out, int32_t* counts, cudaStream_t st) {
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   switch (g.wfmt) {
-    case 0: pack_fill_kernel<0><<<sms * 8, 256, 0, st>>>(g, out, delays, counts); break;
-    case 1: pack_fill_kernel<1><<<sms * 8, 256, 0, st>>>(g, out, delays, counts); break;
-    case 2: pack_fill_kernel<2><<<sms * 8, 256, 0, st>>>(g, out, delays, counts); break;
-    default: pack_fill_kernel<3><<<sms * 8, 256, 0, st>>>(g, out, delays, counts); break;
+    case 0: pack_fill_kernel<0><<<sms * 8, 256, 0, st>>>(g, out, counts); break;
+    case 1: pack_fill_kernel<1><<<sms * 8, 256, 0, st>>>(g, out, counts); break;
+    case 2: pack_fill_kernel<2><<<sms * 8, 256, 0, st>>>(g, out, counts); break;
+    default: pack_fill_kernel<3><<<sms * 8, 256, 0, st>>>(g, out, counts); break;
   }
   return cudaGetLastError();
 }
 
-cudaError_t launch_run_fill(const DevNet& g, uint2* pack, const uint8_t* delays, const int64_t* run_ptr,
-                            uint32_t* runs, ChunkInfo* info, cudaStream_t st) {
+cudaError_t launch_run_fill(const DevNet& g, uint2* pack, const int64_t* run_ptr, uint32_t* runs, ChunkInfo* info,
+                            cudaStream_t st) {
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  run_fill_kernel<<<sms * 8, 256, 0, st>>>(g, pack, delays, run_ptr, runs, info);
+  run_fill_kernel<<<sms * 8, 256, 0, st>>>(g, pack, run_ptr, runs, info);
   return cudaGetLastError();
 }
 
