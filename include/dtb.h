@@ -104,7 +104,9 @@ enum {
  * with four channels and the OU drive), and both keep the ring, without
  * capacities of the caller's, for networks of at most 3,072 neurons and 3,072
  * voxels with at most 200 synapses per neuron and 8,192 in rows of more than 512:
- * they are the faster ones there). */
+ * they are the faster ones there.  A layout so chosen that does not fit the device
+ * memory gives way to the one asked for, and queues of 32-bit weights that do not
+ * fit to the ring). */
 enum {
   DTB_DELIVER_RING = 0,  /* dense ring acc[D][n_channels][N]: every synapse event is one int32
                             reduction into slot (t + d) mod D */

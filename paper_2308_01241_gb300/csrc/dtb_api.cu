@@ -606,7 +606,12 @@ extern "C" {
 
 const char* dtb_last_error(void) { return g_error.c_str(); }
 
-dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
+// The delivery layout of a network: by the rules of size below, as the caller
+// asked, or the ring, which needs the least memory per synapse.
+enum Layout { kLayoutRules, kLayoutAsked, kLayoutRing };
+
+// *chosen: the rules gave another layout than the one asked for.
+static dtb_status create_network(const dtb_network_desc* d, Layout layout, dtb_net** out, bool* chosen) {
   if (!out) return fail(DTB_EINVAL, "out is NULL");
   *out = nullptr;
   if (!d) return fail(DTB_EINVAL, "desc is NULL");
@@ -736,7 +741,7 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
   g.bold_every = d->bold_every;
   g.bold_cap = kBoldLogCap;
   g.log_cap = d->spike_log_capacity > 0 ? d->spike_log_capacity : ((int64_t)1 << 25);
-  g.mode = d->delivery_mode;
+  g.mode = layout == kLayoutRing ? dtb::kModeRing : d->delivery_mode;
   int64_t nnz = 0;
   if (d->csr_on_device) {
     const cudaError_t e = cudaMemcpy(&nnz, d->row_ptr + n, 8, cudaMemcpyDeviceToHost);
@@ -750,7 +755,7 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
   // layouts without capacities of the caller's: the ring for the smallest
   // networks (whose steps run in one CTA), the queues where the accumulator fits
   // the cache
-  const bool free_layout = d->bin_capacity == 0 && d->event_queue_capacity == 0;
+  const bool free_layout = layout == kLayoutRules && d->bin_capacity == 0 && d->event_queue_capacity == 0;
   bool few = dtb::small_network(g) && nnz <= kSmallInDegree * n;
   if (few) {
     std::vector<int64_t> rp;
@@ -772,7 +777,8 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
     g.mode = dtb::kModeRing;
     net->routed = true;
   }
-  if (g.mode == dtb::kModeBins && n <= (int64_t)dtb::kMaxRegions * dtb::kRegionNeurons && d->bin_capacity == 0) {
+  if (g.mode == dtb::kModeBins && n <= (int64_t)dtb::kMaxRegions * dtb::kRegionNeurons && d->bin_capacity == 0 &&
+      layout == kLayoutRules) {
     const bool wide = d->weight_format == DTB_W_INT32 || (g.nch == 4 && d->ou_enable);
     bool room = 4 * npad * g.nch <= (wide ? kQueueMaxBytesWide : kQueueMaxBytes);
     if (room && d->weight_format == DTB_W_INT32) {
@@ -787,6 +793,7 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
       net->routed = true;
     }
   }
+  *chosen = net->routed;
   net->small = g.mode == dtb::kModeRing && few;
   // V, j, ref and I, and the two accumulators of the queue mode
   const int64_t state = npad * (21 + 8 * g.nch + (d->ou_enable ? 4 : 0));
@@ -1144,6 +1151,19 @@ dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
   g.beside = net->beside;
   *out = net;
   return DTB_OK;
+}
+
+dtb_status dtb_create_network(const dtb_network_desc* d, dtb_net** out) {
+  bool chosen = false;
+  dtb_status s = create_network(d, kLayoutRules, out, &chosen);
+  // A layout that does not fit the memory (the caller's allocator may have a
+  // limit of its own) gives way: one of the rules' choice to the one asked for,
+  // and queues of 32-bit weights, which read packed records of 8 bytes per
+  // synapse, to the ring, which reads a delay byte per synapse.
+  if (s == DTB_ENOMEM && chosen) s = create_network(d, kLayoutAsked, out, &chosen);
+  if (s == DTB_ENOMEM && d->delivery_mode == DTB_DELIVER_QUEUE && d->weight_format == DTB_W_INT32)
+    s = create_network(d, kLayoutRing, out, &chosen);
+  return s;
 }
 
 dtb_status dtb_destroy(dtb_net* net) {

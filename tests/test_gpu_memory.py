@@ -57,3 +57,42 @@ def test_creation_needs_no_further_byte_per_synapse(monkeypatch, delivery, bcap,
     np.testing.assert_array_equal(ids, rids)
     for a, b in zip(net.get_state(), ref.get_state()):
         np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("delivery", ["queue", "bins"])
+def test_a_layout_that_does_not_fit_gives_way(monkeypatch, delivery):
+    """32-bit weights under an allocator with less room than the queue layout's
+    packed records (8 bytes per synapse) need, but enough for a delay byte per
+    synapse: the network is created and steps like the oracle.  Less room than the
+    synapse table itself is still DTB_ENOMEM, with everything freed."""
+    from paper_2308_01241_gb300 import dtb
+
+    tb, pull = _tables("int32")
+    csr = dtb.host_csr(tb, pull)
+    nnz = csr[1].size
+    seen = _counting(dtb, monkeypatch)
+    net = dtb.from_tables(tb, csr, delivery="queue", log_capacity=1 << 20)
+    packed = seen["peak"]
+    net.close()
+    assert seen["live"] == 0
+    ref = oracle.OracleNet(ng.oracle_inputs(tb, pull), "f32")
+    seen = _counting(dtb, monkeypatch, limit=packed - 4 * nnz)
+    net = dtb.from_tables(tb, csr, delivery=delivery, log_capacity=1 << 20)
+    assert seen["peak"] <= packed - 4 * nnz
+    total = 0
+    for k in (1, 40, 150):
+        net.step(k)
+        ids, off = net.get_spikes()
+        rids, roff = ref.run(k)
+        total += len(rids)
+        np.testing.assert_array_equal(off, roff)
+        np.testing.assert_array_equal(ids, rids)
+    assert total > 300
+    for a, b in zip(net.get_state(), ref.get_state()):
+        np.testing.assert_array_equal(a, b)
+    net.close()
+    seen = _counting(dtb, monkeypatch, limit=7 * nnz)
+    with pytest.raises(dtb.DtbError) as e:
+        dtb.from_tables(tb, csr, delivery=delivery, log_capacity=1 << 20)
+    assert e.value.code == dtb.DTB_ENOMEM
+    assert seen["live"] == 0
