@@ -659,8 +659,12 @@ struct dtb_mlp {
     mem.push_back(q);
     return q;
   }
-  ~dtb_mlp() {
+  void free_all() {
     for (void* q : mem) cudaFree(q);
+    mem.clear();
+  }
+  ~dtb_mlp() {
+    free_all();
     if (loss) cudaFreeHost(loss);
   }
 };
@@ -847,35 +851,47 @@ dtb_status dtb_mlp_create(int32_t n_in, int32_t width, int32_t depth, int32_t n_
     n->n_params += n->dout[l];
   }
   const size_t P = (size_t)n->n_params;
-  n->fused = width == kW && n_in <= kW && n_out <= kMaxOut && n->nl <= kMaxLayers;
-  n->xs = n->fused ? (n_in + 7) / 8 * 8 : n_in;
-  n->ys = n->fused ? (n_out + 7) / 8 * 8 : n_out;
   int dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&n->sms, cudaDevAttrMultiProcessorCount, dev);
-  bool ok = true;
-  auto A = [&](size_t bytes) { void* q = n->alloc(bytes); if (!q) ok = false; return q; };
-  n->p = (float*)A(4 * P);
-  n->p16 = (bf16*)A(2 * P);
-  n->m = (float*)A(4 * P);
-  n->v = (float*)A(4 * P);
-  n->grad = (float*)A(4 * P);
-  n->x16 = (bf16*)A(2 * (size_t)max_batch * n->xs);
-  n->act.assign(n->nl, nullptr);
-  n->z.assign(n->nl, nullptr);
-  for (int l = 1; l < n->nl; l++) {
-    n->act[l] = (bf16*)A(2 * (size_t)max_batch * width);
-    n->z[l] = (float*)A(4 * (size_t)max_batch * width);
+  auto allocate = [&](bool fused) {
+    bool ok = true;
+    auto A = [&](size_t bytes) { void* q = n->alloc(bytes); if (!q) ok = false; return q; };
+    n->fused = fused;
+    n->xs = fused ? (n_in + 7) / 8 * 8 : n_in;
+    n->ys = fused ? (n_out + 7) / 8 * 8 : n_out;
+    n->p = (float*)A(4 * P);
+    n->p16 = (bf16*)A(2 * P);
+    n->m = (float*)A(4 * P);
+    n->v = (float*)A(4 * P);
+    n->grad = (float*)A(4 * P);
+    n->x16 = (bf16*)A(2 * (size_t)max_batch * n->xs);
+    n->act.assign(n->nl, nullptr);
+    n->z.assign(n->nl, nullptr);
+    for (int l = 1; l < n->nl; l++) {
+      n->act[l] = (bf16*)A(2 * (size_t)max_batch * width);
+      n->z[l] = (float*)A(4 * (size_t)max_batch * width);
+    }
+    n->y = (float*)A(4 * (size_t)max_batch * n_out);
+    n->g.clear();
+    if (fused) {
+      for (int l = 0; l < n->nl - 1; l++) n->g.push_back((bf16*)A(2 * (size_t)max_batch * width));
+    } else {
+      n->g0 = (bf16*)A(2 * (size_t)max_batch * width);
+      n->g1 = (bf16*)A(2 * (size_t)max_batch * width);
+    }
+    n->dy = (bf16*)A(2 * (size_t)max_batch * n->ys);
+    n->part = (float*)A(4 * (size_t)std::max<int64_t>(256, fused ? max_batch / 32 + 1 : 0));
+    return ok;
+  };
+  // The 256-wide path keeps the gradient of every hidden layer, the general one
+  // of two: a batch size for which the former does not fit takes the latter,
+  // with the same results.
+  bool ok = width == kW && n_in <= kW && n_out <= kMaxOut && n->nl <= kMaxLayers && allocate(true);
+  if (!ok) {
+    n->free_all();
+    ok = allocate(false);
   }
-  n->y = (float*)A(4 * (size_t)max_batch * n_out);
-  if (n->fused) {
-    for (int l = 0; l < n->nl - 1; l++) n->g.push_back((bf16*)A(2 * (size_t)max_batch * width));
-  } else {
-    n->g0 = (bf16*)A(2 * (size_t)max_batch * width);
-    n->g1 = (bf16*)A(2 * (size_t)max_batch * width);
-  }
-  n->dy = (bf16*)A(2 * (size_t)max_batch * n->ys);
-  n->part = (float*)A(4 * (size_t)std::max<int64_t>(256, max_batch / 32 + 1));
   if (cudaHostAlloc((void**)&n->loss, sizeof(double), cudaHostAllocDefault) != cudaSuccess) {
     cudaGetLastError();
     n->loss = nullptr;
