@@ -339,9 +339,11 @@ dtb_status dtb_load_state(dtb_net* net, const void* buf, size_t n);
  * word w standing for neuron 32*w + b, every bit at or beyond n zero; d_ids
  * (int32 [n]) receives the ascending ids of the set bits and *d_count (one
  * device int32) their number.  1 <= n < 2^30.  The per-block counts it needs
- * (4 bytes per 1024 neurons + 16) are allocated with cudaMallocAsync on
- * stream and freed there.  Returns after the work is queued and the scratch
- * freed (stream-ordered); DTB_ENOMEM if the allocation fails. */
+ * (4 bytes per 1024 neurons) are allocated on stream and freed there, from a
+ * memory pool of the library's that keeps up to 64 MB on the device, or in a
+ * stream capture from the device's default pool.  Returns after the work is
+ * queued and the scratch freed (stream-ordered); DTB_ENOMEM if the allocation
+ * fails.  Works again after a device reset. */
 dtb_status dtb_spike_compact(const uint32_t* d_bits, int64_t n, int32_t* d_ids, int32_t* d_count, void* stream);
 
 /* One ensemble-Kalman analysis step of the hierarchical mesoscopic data

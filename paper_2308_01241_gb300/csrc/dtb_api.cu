@@ -5,6 +5,7 @@
 // caller's allocator hooks when given), the CUDA graph of a chunk of steps,
 // and copies in and out.  Every step of the simulation itself runs in the
 // kernels of step_kernels.cu.
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -522,42 +523,63 @@ dtb_status check_device_error(dtb_net* net) {
   return fail(DTB_ETIMEOUT, "a bounded wait in the neuron update gave up (TMA copy did not complete)");
 }
 
-// The current device's memory pool for the scratch of dtb_spike_compact (up to
-// 4 MB a call).  The device's default pool gives its memory back at every
-// synchronisation, and the next call then maps it anew: 225 us instead of 44 for
-// the first call after one on the bits of 20M neurons.  This pool keeps what it
-// has, up to 64 MB (it grows by 32 MB); stream order and locking are the driver's.
-cudaError_t scratch_pool(cudaMemPool_t* out) {
-  constexpr int kMaxDevices = 64;
-  static cudaMemPool_t pools[kMaxDevices] = {};
+// The number of the calling thread's context, which no other context of the
+// process gets again; 0 when there is none yet.
+unsigned long long context_id() {
+  typedef CUresult (*GetId)(CUcontext, unsigned long long*);
+  static const GetId get = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    const cudaError_t e = cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess && q == cudaDriverEntryPointSuccess ? (GetId)f : (GetId) nullptr;
+  }();
+  unsigned long long id = 0;
+  return get && get(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+
+// The current context's memory pool for the scratch of dtb_spike_compact (up to
+// 4 MB a call), or NULL.  The device's default pool gives its memory back at
+// every synchronisation, and the next call then maps it anew: 225 us instead of
+// 44 for the first call after one on the bits of 20M neurons.  This pool keeps
+// what it has, up to 64 MB (it grows by 32 MB); stream order and locking are the
+// driver's.  A device reset takes the pool with its context, so pools are kept
+// by the number of their context; the default pool serves beyond kMaxPools.
+cudaMemPool_t scratch_pool() {
+  constexpr int kMaxPools = 64;
+  static struct {
+    unsigned long long ctx;
+    cudaMemPool_t pool;
+  } pools[kMaxPools];
+  static int n_pools = 0;
   static std::mutex mu;
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  const unsigned long long ctx = context_id();
+  if (!ctx) return nullptr;
   std::lock_guard<std::mutex> lk(mu);
-  if (!pools[dev]) {
-    cudaMemPoolProps p{};
-    p.allocType = cudaMemAllocationTypePinned;
-    p.location.type = cudaMemLocationTypeDevice;
-    p.location.id = dev;
-    cudaMemPool_t m = nullptr;
-    // another stream may be under capture, which forbids this call by default
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    e = cudaMemPoolCreate(&m, &p);
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    if (e != cudaSuccess) return e;
-    uint64_t keep = 64ull << 20;
-    e = cudaMemPoolSetAttribute(m, cudaMemPoolAttrReleaseThreshold, &keep);
-    if (e != cudaSuccess) {
-      cudaMemPoolDestroy(m);
-      return e;
-    }
-    pools[dev] = m;
+  for (int k = n_pools - 1; k >= 0; k--)
+    if (pools[k].ctx == ctx) return pools[k].pool;
+  int dev = 0;
+  if (n_pools == kMaxPools || cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+  cudaMemPoolProps p{};
+  p.allocType = cudaMemAllocationTypePinned;
+  p.location.type = cudaMemLocationTypeDevice;
+  p.location.id = dev;
+  cudaMemPool_t m = nullptr;
+  // another stream may be under capture, which forbids this call by default
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  const cudaError_t e = cudaMemPoolCreate(&m, &p);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e != cudaSuccess) return nullptr;
+  uint64_t keep = 64ull << 20;
+  if (cudaMemPoolSetAttribute(m, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+    cudaMemPoolDestroy(m);
+    return nullptr;
   }
-  *out = pools[dev];
-  return cudaSuccess;
+  pools[n_pools].ctx = ctx;
+  pools[n_pools].pool = m;
+  n_pools++;
+  return m;
 }
 
 bool valid_stream(cudaStream_t s) { return s != nullptr && s != cudaStreamLegacy && s != cudaStreamPerThread; }
@@ -1899,7 +1921,7 @@ dtb_status dtb_spike_compact(const uint32_t* d_bits, int64_t n, int32_t* d_ids, 
   // in a stream capture the scratch is the graph's own, from the default pool
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   cudaError_t e = cudaStreamIsCapturing(st, &cap);
-  if (e == cudaSuccess && cap == cudaStreamCaptureStatusNone) e = scratch_pool(&pool);
+  if (e == cudaSuccess && cap == cudaStreamCaptureStatusNone) pool = scratch_pool();
   if (e == cudaSuccess && pool) e = cudaMallocFromPoolAsync(&scratch, dtb::compact_scratch_bytes(n), pool, st);
   if (!scratch) {
     cudaGetLastError();
