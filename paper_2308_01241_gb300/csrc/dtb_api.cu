@@ -112,7 +112,6 @@ struct dtb_net {
   int update_per_sm = 0;     // neuron update CTAs per SM (0 = as many as fit)
   int schedule = -1;         // requested: -1 by size, 0 compaction after the update, 1 beside the next update
   bool small = false;        // a call's steps run in one CTA (launch_small_steps)
-  bool routed = false;       // the layout in use is not the one asked for
   bool beside = false;       // in effect: the compaction of step t runs beside the update of step t + 1
   // the second copy of the spike bits (words) and of the block counts (blocks)
   int64_t flag_par = 0;
@@ -777,6 +776,7 @@ static dtb_status create_network(const dtb_network_desc* d, Layout layout, dtb_n
   // layouts without capacities of the caller's: the ring for the smallest
   // networks (whose steps run in one CTA), the queues where the accumulator fits
   // the cache
+  *chosen = false;
   const bool free_layout = layout == kLayoutRules && d->bin_capacity == 0 && d->event_queue_capacity == 0;
   bool few = dtb::small_network(g) && nnz <= kSmallInDegree * n;
   if (few) {
@@ -797,7 +797,7 @@ static dtb_status create_network(const dtb_network_desc* d, Layout layout, dtb_n
   }
   if (g.mode && free_layout && few) {
     g.mode = dtb::kModeRing;
-    net->routed = true;
+    *chosen = true;
   }
   if (g.mode == dtb::kModeBins && n <= (int64_t)dtb::kMaxRegions * dtb::kRegionNeurons && d->bin_capacity == 0 &&
       layout == kLayoutRules) {
@@ -812,10 +812,9 @@ static dtb_status create_network(const dtb_network_desc* d, Layout layout, dtb_n
     }
     if (room) {
       g.mode = dtb::kModeQueue;
-      net->routed = true;
+      *chosen = true;
     }
   }
-  *chosen = net->routed;
   net->small = g.mode == dtb::kModeRing && few;
   // V, j, ref and I, and the two accumulators of the queue mode
   const int64_t state = npad * (21 + 8 * g.nch + (d->ou_enable ? 4 : 0));
@@ -1940,10 +1939,9 @@ dtb_status dtb_spike_compact(const uint32_t* d_bits, int64_t n, int32_t* d_ids, 
 
 dtb_status dtb_test_preset_counters(dtb_net* net, uint64_t value) {
   if (!net) return fail(DTB_EINVAL, "net is NULL");
-  if (net->g.mode == dtb::kModeRing && !net->routed) return fail(DTB_ESTATE, "the ring mode keeps no event queues");
+  if (net->g.mode == dtb::kModeRing) return fail(DTB_ESTATE, "the ring layout in use keeps no event queues");
   const uint64_t cap = (uint64_t)std::max<int64_t>(net->g.qcap, net->g.mode == dtb::kModeBins ? net->g.bcap : 0);
   if (value < cap || value > ((uint64_t)1 << 62)) return fail(DTB_EINVAL, "value out of capacity .. 2^62");
-  if (net->g.mode == dtb::kModeRing) return DTB_OK;  // a layout without counters was chosen
   DTB_CUDA(dtb::launch_preset_counters(net->g, (unsigned long long)value, net->stream));
   DTB_CUDA(cudaStreamSynchronize(net->stream));
   return DTB_OK;
