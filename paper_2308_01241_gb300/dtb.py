@@ -228,13 +228,17 @@ def dtb_spike_compact_noalloc(bits, n: int, ids, count, stream=None) -> None:
 
 
 class _TorchAllocator:
-    """Device memory for the library from torch's caching allocator."""
+    """Device memory for the library from torch's caching allocator.
 
-    def __init__(self, device):
+    A block it hands out may have been freed with work on it still queued on
+    torch's current stream, so the library's stream waits for that work."""
+
+    def __init__(self, device, stream):
         import torch
 
         self.torch = torch
         self.device = torch.device(device)
+        self.stream = stream
         self.live = {}
         self.alloc_cb = ALLOC_FN(self._alloc)
         self.free_cb = FREE_FN(self._free)
@@ -242,6 +246,7 @@ class _TorchAllocator:
     def _alloc(self, nbytes, ctx):
         try:
             t = self.torch.empty(int(nbytes), dtype=self.torch.uint8, device=self.device)
+            self.stream.wait_stream(self.torch.cuda.current_stream(self.device))
         except Exception:
             return None
         p = t.data_ptr()
@@ -268,7 +273,7 @@ class Network:
         self.torch = torch
         self.device = torch.device(device)
         self.stream = torch.cuda.Stream(device=self.device)
-        self._alloc = _TorchAllocator(self.device)
+        self._alloc = _TorchAllocator(self.device, self.stream)
         self._keep = []
         bold = bold or {}
         self.n, self.n_vox, self.n_ch, self.D = int(n), len(voxel_start) - 1, int(n_ch), int(d_max) + 1
@@ -290,6 +295,7 @@ class Network:
         on_dev = not isinstance(csr[0], np.ndarray)
         if on_dev:
             keep.extend(csr)
+            torch.cuda.current_stream(self.device).synchronize()  # creation reads them on other streams
             d.row_ptr, d.syn_word, d.syn_w = (c.data_ptr() for c in csr[:3])
             d.row_shift = csr[3].data_ptr() if len(csr) > 3 and csr[3] is not None else None
         else:
