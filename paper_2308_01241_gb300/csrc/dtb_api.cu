@@ -355,7 +355,7 @@ dtb::DevNet step_view(const dtb_net* net, int32_t t_rel) {
   if (t_rel & 1) {
     d.flags += net->flag_par;
     d.blk_cnt += net->cnt_par;
-    d.blk_items += net->cnt_par;
+    if (d.blk_items) d.blk_items += net->cnt_par;
   }
   return d;
 }
@@ -894,7 +894,7 @@ static dtb_status create_network(const dtb_network_desc* d, Layout layout, dtb_n
   net->cnt_par = (g.nblk + 3) & ~3;  // keeps the second copy 16-byte aligned
   g.flags = (uint32_t*)A(2 * (npad / 8));
   g.blk_cnt = (int32_t*)A(8 * (size_t)net->cnt_par);
-  g.blk_items = (int32_t*)A(8 * (size_t)net->cnt_par);
+  if (g.mode == dtb::kModeBins) g.blk_items = (int32_t*)A(8 * (size_t)net->cnt_par);
   g.n_items = (int32_t*)A(16);
   g.spk = (int32_t*)A(8 * npad);  // two copies, as the counts and the log's position
   g.spk_par = npad;
@@ -1109,8 +1109,9 @@ static dtb_status create_network(const dtb_network_desc* d, Layout layout, dtb_n
     g.syn_delay = sd;
   }
 
-  // work items per neuron (one byte each), streamed with the neuron update's tiles
-  {
+  // bins mode: work items per neuron (one byte each), streamed with the neuron
+  // update's tiles
+  if (g.mode == dtb::kModeBins) {
     uint8_t* ni = (uint8_t*)net->dalloc((size_t)npad);
     if (!ni) {
       delete net;
