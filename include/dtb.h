@@ -232,8 +232,8 @@ dtb_status dtb_get_state(dtb_net* net, float* V, float* j, uint8_t* ref, int32_t
 
 /* Overwrites the state (checkpoint restore, tests); NULL leaves a part
  * unchanged; arrays as in dtb_get_state; t >= 0 (else DTB_EINVAL).  In the
- * queue mode the ring is turned back into queues (a temporary allocation as
- * in dtb_get_state), in the bins mode it goes into the spill ring.  The spike
+ * queue and bins modes the ring goes into the spill ring, and a ring left
+ * unchanged keeps its slots (slot t mod D of the new t is next).  The spike
  * log of the last dtb_step call is then empty (no steps). */
 dtb_status dtb_set_state(dtb_net* net, const float* V, const float* j, const uint8_t* ref, const int32_t* ring,
                          int64_t t);
@@ -306,9 +306,9 @@ dtb_status dtb_set_launch_shapes(dtb_net* net, int32_t update_stages, int32_t up
  *      and before that of step t + 1, on the update's stream;
  *   1: the compaction of step t runs beside the neuron update of step t + 1
  *      (the two use alternate copies of the spike bits and block counts), on
- *      the delivery's stream;
- *  -1: chosen by size (the default): 1 for networks of at most 4,096 blocks of
- *      1,024 neurons, whose kernels leave most of the GPU idle, else 0.
+ *      the delivery's stream with bins, else on the BOLD step's;
+ *  -1: chosen by size (the default): 1 for networks of at most 6,144 blocks of
+ *      1,024 neurons, else 0.
  * DTB_EINVAL for other values.  Results do not depend on the schedule: every
  * kernel reads and writes what it does in the plain order of the step (the
  * paper's per-step sequence of update, spike collection and delivery, §V.B).
@@ -441,8 +441,7 @@ dtb_status dtb_assimilate(dtb_ensemble* ens, const float* bold_obs, int32_t n_tr
  * library's device code, so make that first call before any stream capture.
  * All calls share the one array, so calls that overlap on
  * the GPU (different streams, or different host threads, at the same time)
- * race and corrupt each other's results; serialise them.  The parts that
- * must start at zero are cleared by every call. */
+ * race and corrupt each other's results; serialise them. */
 dtb_status dtb_spike_compact_noalloc(const uint32_t* d_bits, int64_t n, int32_t* d_ids, int32_t* d_count,
                                      void* stream);
 

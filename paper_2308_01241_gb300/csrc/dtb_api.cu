@@ -4,7 +4,7 @@
 // once to float), Poisson inversion thresholds, device memory (through the
 // caller's allocator hooks when given), the CUDA graph of a chunk of steps,
 // and copies in and out.  Every step of the simulation itself runs in the
-// kernels of step_kernels.cu.
+// kernels of step_kernels.cu, deliver.cu and bins.cu.
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -51,8 +51,8 @@ constexpr int64_t kSmallSteps = 4096;  // steps per launch of a small network (s
 // and the more spikes.  3,000 neurons at 8 Hz, us per step of the launches and of
 // the one CTA: 7.6 and 4.3 with 150 synapses per neuron, 7.7 and 4.7 with 200,
 // 7.8 and 5.9 with 300 (in 40 voxels 8.7 and 9.5), 8.6 and 13.5 with 1,000.
-// At 150 the two meet near 100 Hz; 1,000 neurons: 6.8 and 3.3 at 10 Hz, 9.5 and
-// 7.9 at 117 Hz.
+// 3,000 neurons with 200 synapses meet near 80 Hz; 1,000 neurons: 6.8 and 3.3 at
+// 10 Hz, 9.5 and 7.9 at 117 Hz.
 constexpr int64_t kSmallInDegree = 200;
 // Synapses of such a network in rows of more than a delivery work item: a long row
 // holds up its warp, and with it every step in which its neuron fires.  3,000
@@ -79,11 +79,17 @@ constexpr int64_t kKeepBytes = (int64_t)88 << 20;
 // of the caller's): it stays in the L2 cache beside the neuron state, and one
 // reduction there per event is less work than sorting the events into bins.
 // us a step, bins and queue: 36.4 and 29.8 (2M neurons, 15 Hz), 49.3 and 47.2
-// (3.6M, 7 Hz), 87.4 and 79.5 (3.6M int8, 30 Hz); 51.7 and 56.7 (3.9M, 7 Hz), 61.3
-// and 68.5 (5M, 7 Hz): the accumulators no longer fit.  The bins' kernels are
-// slower with 32-bit weights (8-byte events) and for four channels with the OU
-// drive, where the line lies further out: 87.3 and 68.5 (5M int32, 7 Hz), 195 and
-// 104 (30 Hz), 91.3 and 80.4 (6M int32), 115 and 94 (3M, four channels, OU, 30 Hz).
+// (3.6M, 7 Hz), 87.4 and 79.5 (3.6M int8, 30 Hz).  Beyond, the accumulators no
+// longer fit, and it depends on the rate: at 7, 15 and 30 Hz 49.6 and 51.4, 61.9 and
+// 64.8, 85.8 and 81.8 (3.9M); 55.5 and 60.7, 69.3 and 75.3, 95.1 and 93.9 (4.5M); 61.0
+// and 68.2, 77.9 and 83.6, 105.8 and 104.2 (5M).  Four channels: 31.7 and 31.0, 38.3
+// and 38.1, 50.7 and 46.9 (1.8M); at 7 and 30 Hz 33.1 and 35.8, 57.6 and 53.8 (2M),
+// 43.6 and 51.1, 77.9 and 81.0 (2.9M).  The OU drive: 66.0 and 61.8, 92.2 and 87.1
+// (3.6M); 67.4 and 69.2, 105 and 96.7 (4M).
+// The bins' kernels are slower with 32-bit weights (8-byte events) and for four
+// channels with the OU drive, where the line lies further out: at 7 and 30 Hz 73.4
+// and 52.4, 155 and 83.0 (4M int32), 101.7 and 86.7, 240 and 132 (6.2M int32), 60.7
+// and 45.6, 80.6 and 61.5 (2M, four channels, OU), 77.7 and 69.8, 120 and 95.8 (3.1M).
 constexpr int64_t kQueueMaxBytes = 28 << 20, kQueueMaxBytesWide = 48 << 20;
 constexpr int kBoldLogCap = 1024;
 
@@ -1152,7 +1158,10 @@ static dtb_status create_network(const dtb_network_desc* d, Layout layout, dtb_n
   // chunks each when the network fires at 30 Hz, since each CTA without work
   // costs its launch (us a step with 1 and 8 per SM: 50k neurons 8.4 and 10.2,
   // 200k with four channels 10.9 and 12.1; 1M at 15 Hz 19.6 with 5, 20.1 with 8;
-  // 2M 33.4 with 4, 32.4 with 8).
+  // 2M 33.4 with 4, 32.4 with 8).  It serves higher rates too, us a step with this
+  // rule and with 8: 50k neurons 9.5 and 9.8 at 67 Hz, 11.7 and 13.1 at 249 Hz; 200k
+  // 12.5 and 13.6 at 93 Hz, 15.6 and 17.9 at 292 Hz; 1M 22.7 and 24.4 at 67 Hz, 41.0
+  // and 43.8 at 249 Hz.
   // In ring mode two at most: its reductions miss the cache and hold up the
   // neuron update beside them (us a step with 1, 2, 3 and 8: 2M at 15 Hz 38.5,
   // 41.2, 42.5, 42.6; 2M at 30 Hz 67.1, 66.1, 66.5, 68.2; 1.3M at 30 Hz 44.6,

@@ -762,8 +762,8 @@ __device__ __forceinline__ int block_excl_scan(int x, int* s, int* total) {
 // thread walks a chain of lookups per spike or per item, so a tile with a
 // crowded word or a row of many items costs a few memory latencies, not one
 // per spike.
-// In the queue mode the delivery reads the spike bits itself and no work items
-// are built.
+// In the queue and ring modes the update lists the delivery's work and no work
+// items are built here.
 //
 // BESIDE: the instance of the networks whose compaction runs beside an update,
 // with the update's division of an SM's memory; the other keeps its own, which
