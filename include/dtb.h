@@ -104,7 +104,8 @@ enum {
  * with four channels and the OU drive), and both keep the ring, without
  * capacities of the caller's, for networks of at most 3,072 neurons and 3,072
  * voxels with at most 200 synapses per neuron and 8,192 in rows of more than 512:
- * they are the faster ones there.  A layout so chosen that does not fit the device
+ * they are the faster ones there (steps of such networks run in one CTA, or as the
+ * others' if the last call's activity was high).  A layout so chosen that does not fit the device
  * memory gives way to the one asked for, and queues of 32-bit weights that do not
  * fit to the ring). */
 enum {

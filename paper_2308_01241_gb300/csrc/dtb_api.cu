@@ -61,6 +61,14 @@ constexpr int64_t kSmallInDegree = 200;
 // 30,000 (103 Hz), 7.0 and 27 with ten of 30,000, 7.1 and 22 with a hundred of
 // 3,000 (74 Hz).
 constexpr int64_t kSmallLongRows = 8192;
+// Row parts of 128 synapses that a warp of the one CTA delivers per step (a row of
+// one part counts 0.75), above which the next call of such a network takes the
+// launches, and below which the one CTA again.  us a step of the one CTA and of
+// the launches, 3,000 neurons: 6.7 and 7.0 at 74 Hz (200 synapses, 1.4 parts), 6.7 and
+// 7.2 at 86 Hz (150, 1.6), 8.5 and 7.5 at 107 Hz (200, 2.0), 14.4 and 8.6 at 245 Hz
+// (200, 4.6), 7.1 and 8.4 at 238 Hz (50, 1.7), 8.7 and 8.7 at 312 Hz (50, 2.2); 1,000
+// neurons: 5.5 and 6.4 at 123 Hz (150, 1.5), 8.6 and 7.2 at 266 Hz (150, 3.3).
+constexpr double kSmallPartsOff = 1.9, kSmallPartsOn = 1.7;
 constexpr int kTimedKernels = 5;  // update, compaction, delivery, drain or binning, BOLD
 // Networks of at most this many 1,024-neuron blocks run the compaction of a
 // step beside the neuron update of the next by default: their kernels leave
@@ -117,7 +125,11 @@ struct dtb_net {
   int update_stages = 3;     // neuron update pipeline depth
   int update_per_sm = 0;     // neuron update CTAs per SM (0 = as many as fit)
   int schedule = -1;         // requested: -1 by size, 0 compaction after the update, 1 beside the next update
-  bool small = false;        // a call's steps run in one CTA (launch_small_steps)
+  bool few = false;          // its steps may run in one CTA (launch_small_steps)
+  bool small = false;        // the next call's do
+  double small_parts = 0;    // few: row parts per warp of that CTA and spike
+  int64_t seen_t = 0;        // few: step and spike count of the last look at the activity (seen_t < 0: none)
+  unsigned long long seen_spikes = 0;
   bool beside = false;       // in effect: the compaction of step t runs beside the update of step t + 1
   // the second copy of the spike bits (words) and of the block counts (blocks)
   int64_t flag_par = 0;
@@ -296,6 +308,8 @@ dtb_status init_state(dtb_net* net) {
   DTB_CUDA(cudaMemcpyAsync(g.bold, bold.data(), bold.size() * 4, cudaMemcpyHostToDevice, st));
   DTB_CUDA(cudaStreamSynchronize(st));
   net->t = 0;
+  net->seen_t = 0;
+  net->seen_spikes = 0;
   net->call_t0 = 0;
   net->call_steps = 0;
   return DTB_OK;
@@ -520,10 +534,21 @@ namespace {
 
 // The kernels' error word: a bounded wait that gave up (the state of that
 // step is incomplete, the call reports DTB_ETIMEOUT and the word is cleared).
+// A small network's activity comes along: it decides where the next call's steps
+// run (both ways give the same state, bit for bit).
 dtb_status check_device_error(dtb_net* net) {
-  int32_t err = 0;
-  DTB_CUDA(cudaMemcpy(&err, net->g.err, 4, cudaMemcpyDeviceToHost));
-  if (err == 0) return DTB_OK;
+  struct {
+    int32_t err, pad[3];
+    unsigned long long spikes;  // g.spikes lies 16 bytes behind g.err
+  } w{};
+  DTB_CUDA(cudaMemcpy(&w, net->g.err, sizeof(w), cudaMemcpyDeviceToHost));
+  if (net->few && net->seen_t >= 0 && net->t > net->seen_t) {
+    const double parts = net->small_parts * (double)(w.spikes - net->seen_spikes) / (double)(net->t - net->seen_t);
+    net->small = parts <= (net->small ? kSmallPartsOff : kSmallPartsOn);
+  }
+  net->seen_t = net->t;
+  net->seen_spikes = w.spikes;
+  if (w.err == 0) return DTB_OK;
   DTB_CUDA(cudaMemset(net->g.err, 0, 4));
   return fail(DTB_ETIMEOUT, "a bounded wait in the neuron update gave up (TMA copy did not complete)");
 }
@@ -821,7 +846,9 @@ static dtb_status create_network(const dtb_network_desc* d, Layout layout, dtb_n
       *chosen = true;
     }
   }
-  net->small = g.mode == dtb::kModeRing && few;
+  net->few = net->small = g.mode == dtb::kModeRing && few;
+  const double parts = std::ceil((double)nnz / (double)n / 128.0);
+  net->small_parts = (parts > 1.0 ? parts : 0.75) / (double)dtb::small_warps(g);
   // V, j, ref and I, and the two accumulators of the queue mode
   const int64_t state = npad * (21 + 8 * g.nch + (d->ou_enable ? 4 : 0));
   g.keep_state = g.mode == dtb::kModeQueue && state <= kKeepBytes;
@@ -910,9 +937,9 @@ static dtb_status create_network(const dtb_network_desc* d, Layout layout, dtb_n
   g.log_pos = (int64_t*)A(16);
   g.call_steps = (int32_t*)A(16);
   g.log_trunc = (int32_t*)A(16);
-  g.err = (int32_t*)A(16);
+  g.err = (int32_t*)A(32);
   g.events = (unsigned long long*)A(16);
-  g.spikes = (unsigned long long*)A(16);
+  if (g.err) g.spikes = (unsigned long long*)((char*)g.err + 16);
   g.bold = (float*)A(4 * 5 * (size_t)nv);
   g.vox_spikes = (unsigned long long*)A(8 * (size_t)nv);
   g.bold_log = (float*)A(4 * (size_t)kBoldLogCap * nv);
@@ -1430,6 +1457,7 @@ dtb_status dtb_set_state(dtb_net* net, const float* V, const float* j, const uin
   DTB_CUDA(cudaMemcpyAsync(g.t_base, &t, 8, cudaMemcpyHostToDevice, st));
   DTB_CUDA(cudaStreamSynchronize(st));
   net->t = t;
+  net->seen_t = -1;
   net->call_steps = 0;
   return DTB_OK;
 }

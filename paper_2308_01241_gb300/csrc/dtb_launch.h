@@ -27,6 +27,7 @@ cudaError_t launch_begin_call(const DevNet& g, cudaStream_t st);
 // Networks of a few blocks in ring mode: n_steps whole steps in one CTA (the
 // step counter moves on, the spike log grows).
 bool small_network(const DevNet& g);
+int small_warps(const DevNet& g);  // of that CTA
 cudaError_t launch_small_steps(const DevNet& g, int32_t n_steps, cudaStream_t st);
 int deliver_blocks_per_sm();
 // Attributes of the step's kernels on the current device (once per network).

@@ -1322,6 +1322,8 @@ cudaError_t launch_neuron_update(const DevNet& g, int32_t t_rel, cudaStream_t st
 // counts have room in shared memory for one voxel per neuron.
 bool small_network(const DevNet& g) { return g.nblk <= kSmallBlocks && g.nv <= SmallSmem::kN; }
 
+int small_warps(const DevNet& g) { return g.nblk == 1 ? 16 : 32; }
+
 cudaError_t launch_small_steps(const DevNet& g, int32_t n_steps, cudaStream_t st) {
   static DeviceLaunch cache[kMaxDevices];
   static std::mutex mu;
@@ -1340,7 +1342,7 @@ cudaError_t launch_small_steps(const DevNet& g, int32_t n_steps, cudaStream_t st
   if (e != cudaSuccess) return e;
   const size_t smem = SmallSmem::bytes(g.nv);
   const bool few = g.nblk == 1;  // half the threads with twice the registers each, none of them spilled
-  auto run = [&](auto kernel) { kernel<<<1, few ? 512 : 1024, smem, st>>>(g, n_steps); };
+  auto run = [&](auto kernel) { kernel<<<1, 32 * small_warps(g), smem, st>>>(g, n_steps); };
   if (g.nch == 2) {
     if (g.ou) few ? run(small_steps_kernel<2, true, 512>) : run(small_steps_kernel<2, true, 1024>);
     else few ? run(small_steps_kernel<2, false, 512>) : run(small_steps_kernel<2, false, 1024>);
