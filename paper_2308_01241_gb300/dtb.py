@@ -231,7 +231,8 @@ class _TorchAllocator:
     """Device memory for the library from torch's caching allocator.
 
     A block it hands out may have been freed with work on it still queued on
-    torch's current stream, so the library's stream waits for that work."""
+    torch's current stream, so the library's stream waits for that work: once
+    for all of a network's creation, then at every allocation."""
 
     def __init__(self, device, stream):
         import torch
@@ -239,6 +240,7 @@ class _TorchAllocator:
         self.torch = torch
         self.device = torch.device(device)
         self.stream = stream
+        self.created = False
         self.live = {}
         self.alloc_cb = ALLOC_FN(self._alloc)
         self.free_cb = FREE_FN(self._free)
@@ -246,7 +248,8 @@ class _TorchAllocator:
     def _alloc(self, nbytes, ctx):
         try:
             t = self.torch.empty(int(nbytes), dtype=self.torch.uint8, device=self.device)
-            self.stream.wait_stream(self.torch.cuda.current_stream(self.device))
+            if self.created:
+                self.wait()
         except Exception:
             return None
         p = t.data_ptr()
@@ -255,6 +258,11 @@ class _TorchAllocator:
 
     def _free(self, p, ctx):
         self.live.pop(p, None)
+
+    def wait(self):
+        current = self.torch.cuda.current_stream(self.device)
+        if not current.query():  # idle, as it mostly is between calls: nothing to wait for
+            self.stream.wait_stream(current)
 
 
 class Network:
@@ -325,7 +333,9 @@ class Network:
         if ou:
             d.ou_enable, d.ou_mu, d.ou_sigma, d.ou_tau = 1, float(ou["mu"]), float(ou["sigma"]), float(ou["tau"])
         with torch.cuda.device(self.device):
+            self._alloc.wait()
             self.h = dtb_create_network(d)
+        self._alloc.created = True
         self._keep = [k for k in keep if not isinstance(k, np.ndarray)]  # host arrays were copied
 
     # -- lifecycle
