@@ -39,7 +39,8 @@ dtb_status dtb_mlp_create(int32_t n_in, int32_t width, int32_t depth, int32_t n_
                           const float* params, dtb_mlp** out);
 dtb_status dtb_mlp_destroy(dtb_mlp* mlp);
 
-/* Inference: d_x [B][n_in] FP32 device -> d_y [B][n_out] FP32 device. */
+/* Inference: d_x [B][n_in] FP32 device -> d_y [B][n_out] FP32 device, which may
+ * overlap d_x. */
 dtb_status dtb_mlp_forward(dtb_mlp* mlp, const float* d_x, float* d_y, int64_t B, void* stream);
 
 /* Loss and gradients of the mean squared error to targets d_t [B][n_out]:

@@ -51,4 +51,4 @@ def test_a_look_at_the_queues_is_quick():
             net.get_ring_at(idx)
             t.append(time.perf_counter() - t0)
         us.append(np.median(t) * 1e6)
-    assert us[1] < us[0] + 100, us
+    assert us[1] < us[0] + 120, us
