@@ -1427,7 +1427,7 @@ dtb_status dtb_set_state(dtb_net* net, const float* V, const float* j, const uin
     // in slot by slot; queues, and the accumulator or the bins, start empty
     const size_t bytes = 4 * (size_t)g.D * g.nch * np;
     std::vector<int32_t> dirty((size_t)g.D);
-    for (int64_t x = t; x < t + g.D; x++) dirty[(size_t)(x % g.D)] = dtb::spill_mark(x);  // the steps to come
+    for (int32_t k = 0; k < g.D; k++) dirty[(size_t)((t % g.D + k) % g.D)] = dtb::spill_mark(t, k);  // the steps to come
     cudaError_t e = cudaMemsetAsync(g.spill, 0, bytes, st);
     if (e == cudaSuccess)
       e = cudaMemcpy2DAsync(g.spill, 4 * np, ring, 4 * n, 4 * n, (size_t)g.D * g.nch, cudaMemcpyHostToDevice, st);
@@ -1446,9 +1446,10 @@ dtb_status dtb_set_state(dtb_net* net, const float* V, const float* j, const uin
     std::vector<int32_t> old((size_t)g.D), mark((size_t)g.D, 0);
     DTB_CUDA(cudaMemcpyAsync(old.data(), g.spill_dirty, 4 * (size_t)g.D, cudaMemcpyDeviceToHost, st));
     DTB_CUDA(cudaStreamSynchronize(st));
-    for (int64_t x = t; x < t + g.D; x++) {
-      const int64_t s = x % g.D, was = net->t + (s - net->t % g.D + g.D) % g.D;
-      if (old[(size_t)s] == dtb::spill_mark(was)) mark[(size_t)s] = dtb::spill_mark(x);
+    for (int32_t k = 0; k < g.D; k++) {
+      const int64_t s = (t % g.D + k) % g.D;
+      const int32_t was = (int32_t)((s - net->t % g.D + g.D) % g.D);
+      if (old[(size_t)s] == dtb::spill_mark(net->t, was)) mark[(size_t)s] = dtb::spill_mark(t, k);
     }
     DTB_CUDA(cudaMemcpyAsync(g.spill_dirty, mark.data(), 4 * (size_t)g.D, cudaMemcpyHostToDevice, st));
     DTB_CUDA(cudaStreamSynchronize(st));  // mark leaves scope

@@ -357,7 +357,10 @@ __device__ __forceinline__ int32_t decode_weight(uint32_t code, int32_t wfmt, in
   return (int32_t)(signed char)(code & 0xFFu) * (1 << (code >> 8));
 }
 
-__host__ __device__ __forceinline__ int32_t spill_mark(int64_t arrival) { return (int32_t)(uint32_t)(arrival + 1); }
+// The mark of spilled events that arrive `later` steps after a step.
+__host__ __device__ __forceinline__ int32_t spill_mark(int64_t step, int32_t later = 0) {
+  return (int32_t)((uint32_t)step + (uint32_t)later + 1u);
+}
 
 // Voxel of neuron i: coarse table entry, then a forward scan of voxel starts.
 __device__ __forceinline__ int32_t voxel_of(const DevNet& g, int32_t i) {

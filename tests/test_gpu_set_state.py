@@ -10,8 +10,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("delivery,qcap,bcap", [("queue", 1024, 0), ("bins", 1024, 20000)])
-@pytest.mark.parametrize("move", [8, -2])
-def test_spilled_events_follow_a_moved_step(delivery, qcap, bcap, move):
+@pytest.mark.parametrize("move,far", [(8, False), (-2, False), (8, True)])
+def test_spilled_events_follow_a_moved_step(delivery, qcap, bcap, move, far):
     from paper_2308_01241_gb300 import dtb
 
     tb = ng.make_tables(dict(ng.load_config("c2_multi_voxel_1m"), gain={"default": 1.45}), n_neurons=200003, n_vox=24,
@@ -28,6 +28,8 @@ def test_spilled_events_follow_a_moved_step(delivery, qcap, bcap, move):
     moved = t + move * 2 * D
     assert moved >= 0
     ref.set_state(V, j, r, ring, moved)
+    if far:  # by way of the last step there is
+        net.set_state(t=2 ** 63 - 1)
     net.set_state(t=moved)
     for k in (1, 2 * D, 40):
         net.step(k)
